@@ -23,7 +23,7 @@ enum DevErr : int32_t {
     kDevLevelOverflow = 5,
     kDevBucketOverflow = 6,
     kDevCancelled = 7,
-    kDevWide = 8,  // weighted source kernel: a count or distance needs the 16-byte pairs
+    kDevWide = 8,  // a count (or weighted distance) does not fit its narrow form: rerun with the wide one
 };
 
 // Per-launch control block of the persistent traversal kernel.
@@ -44,6 +44,15 @@ struct Counters {
     unsigned long long eb;         // sum over tiles of the out-arcs of those vertices
     unsigned long long vpairs;     // vertex scan: (t, s) pairs with the query vertex on a shortest s-t path
     unsigned long long pull_levels; // forward levels run bottom-up (pull over R(G))
+    unsigned long long tiles_taken; // tiles handed out after each team's first
+};
+
+// Barrier words of one team of blocks (unweighted traversal), and its next
+// tile; a cache line each.
+struct __align__(128) TeamBar {
+    uint32_t count;
+    uint32_t gen;
+    unsigned long long next;
 };
 
 // One unit of expansion work: arcs [a0, a0 + na) of vertex v, the k-th of
@@ -85,7 +94,7 @@ struct TravParams {
     int32_t vs_stride;  // words per vertex
     int32_t pad0;
     int32_t *tag;       // [n] last level a vertex was appended at, -1 none
-    double *sigma;      // [n * S] sigma, then c = (1 + delta) / sigma in place
+    double *sigma;      // [n * S] sigma (unweighted: 32-bit counts, or fp64 after an overflow; weighted: then c in place)
     double *acc;        // [n * S] backward sums of c over tight out-arcs (unweighted), zero between levels
     // level history
     int32_t *hv;        // [hcap]
@@ -93,14 +102,14 @@ struct TravParams {
     uint16_t *hs;       // [hcap] source slot of an entry (weighted)
     int64_t hcap;
     Chunk *chunks;      // [ccap]
-    Chunk *ichunks;     // [ccap] in-arc (R(G)) chunks of the entries, per level (unweighted SPD)
+    Chunk *ichunks;     // [ccap] in-arc (R(G)) chunks of the entries, per level (unweighted)
     int64_t ccap;
     double *partial;    // [pcap * S]
     int32_t *pdone;     // [pcap]
     int64_t pcap;
     unsigned long long *lev_cnt;   // [maxlev + 2]
     unsigned long long *lev_ccnt;  // [maxlev + 2]
-    unsigned long long *lev_grab;  // [2 * (maxlev + 2)] chunk hand-out counters, forward then backward
+    unsigned long long *lev_grab;  // [6 * (maxlev + 2)] hand-out counters and counts, see bcd_workspace
     int64_t *lev_start;            // [maxlev + 2]
     int64_t *lev_cstart;           // [maxlev + 2]
     int64_t *lev_icstart;          // [maxlev + 2] first in-arc chunk of each level
@@ -163,6 +172,14 @@ struct TravParams {
     uint64_t *rvmask;        // [n]
     int32_t *levout;         // [n] level of first discovery (reach mode, one root), or NULL
     Counters *ctr;
+    // unweighted: the grid's blocks form nteams teams of team_blocks, each with
+    // the state of one tile (the arrays above are those of team 0)
+    TeamBar *bar;
+    int32_t nteams;
+    int32_t team_blocks;
+    int64_t hm_words;        // words of hm per team
+    int32_t ws_slots;        // source slots the state arrays are sized for
+    int32_t pad4;
     double timeout_ns;
     const int32_t *cancel;   // host-mapped flag, non-zero: leave at the next tile start (may be NULL)
 };
@@ -175,6 +192,8 @@ struct TravParams {
 
 struct bcd_workspace {
     int W = 0;           // mask words per tile (S = 64 W sources)
+    int teams = 1;       // tiles whose state is held at once (unweighted): the arrays of state below hold that many
+    bcd::TeamBar *bar = nullptr;  // [teams]
     int64_t n = 0;
     int64_t m = 0;
     // dense state
@@ -182,7 +201,10 @@ struct bcd_workspace {
     int vs_stride = 0;
     int32_t *tag = nullptr;
     double *sigma = nullptr;
-    double *acc = nullptr;        // [n * 64 * W] unweighted graphs
+    size_t sigma_bytes = 8;       // bytes per count (4: 32-bit counts of unweighted graphs)
+    bool sigma_zero = false;      // the slab is all zero
+    int64_t sigma_key = -1;       // unweighted: row width, count type and chunk_arcs the slab was last used with
+    double *acc = nullptr;        // [n * 64 * W] unweighted graphs, from the first Eq. 4 launch on
     // history
     int32_t *hv = nullptr;
     uint64_t *hm = nullptr;
@@ -198,7 +220,7 @@ struct bcd_workspace {
     unsigned long long *lev_cnt = nullptr;
     unsigned long long *lev_ccnt = nullptr;
     unsigned long long *lev_grab = nullptr;  // [6 * (maxlev + 2)]: forward and backward hand-out, in-arc chunk
-                                             // counts, frontier out-arc sums, entries | chunks << 32
+                                             // counts, frontier out-arc sums, entries | chunks << 32, gather hand-out
     int64_t *lev_start = nullptr;
     int64_t *lev_cstart = nullptr;
     int64_t *lev_icstart = nullptr;
@@ -239,7 +261,7 @@ struct bcd_workspace {
     unsigned long long *sds = nullptr;     // [sblocks * n * 2]: (distance, sigma) of each vertex
     uint32_t *stb = nullptr;               // [sblocks * (m + 31) / 32]: tight-candidate arc bits
     int32_t slayout = 0;                   // how sds is cleared: 1 16-byte pairs, 2 8-byte words
-    bool swide = false;                    // a narrow launch overflowed: 16-byte pairs from now on
+    bool swide = false;                    // a narrow launch overflowed: 16-byte pairs (unweighted: fp64 counts) from now on
     int32_t *shv = nullptr;                // [sblocks * n]
     int32_t *slstart = nullptr;            // [sblocks * smaxlev]
     unsigned long long *sldist = nullptr;  // [sblocks * smaxlev]

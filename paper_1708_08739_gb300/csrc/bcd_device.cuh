@@ -27,24 +27,27 @@ __device__ __forceinline__ unsigned long long ld_vol(const unsigned long long *p
 
 __device__ __forceinline__ void set_err(Counters *c, int32_t code) { atomicCAS(&c->err, 0, code); }
 
-// Grid-wide barrier for a cooperative launch. Every wait is bounded by
-// timeout_ns of wall time (and a spin cap); on timeout or when another block
-// has flagged an error, returns false and the caller leaves the kernel.
-__device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_ns) {
+// Barrier of nb blocks of a cooperative launch, on the words count and gen.
+// Every wait is bounded by timeout_ns of wall time (and a spin cap); on
+// timeout or when another block has flagged an error, returns false and the
+// caller leaves the kernel.
+__device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_ns, uint32_t *count, uint32_t *gens,
+                                    uint32_t nb) {
     __shared__ int s_err;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const uint32_t nb = gridDim.x;
-        const uint32_t arrived = atomicAdd(&c->bar_count, 1u);
+        const uint32_t arrived = nb > 1 ? atomicAdd(count, 1u) : 0u;
         if (arrived == nb - 1) {
-            atomicExch(&c->bar_count, 0u);
-            __threadfence();
-            atomicExch(&c->bar_gen, gen + 1);
+            if (nb > 1) {
+                atomicExch(count, 0u);
+                __threadfence();
+                atomicExch(gens, gen + 1);
+            }
         } else {
             const unsigned long long t0 = global_ns();
             unsigned long long spins = 0;
-            while (ld_acquire(&c->bar_gen) == gen) {
+            while (ld_acquire(gens) == gen) {
                 if (ld_vol(&c->err) != 0) break;
                 ++spins;
                 if ((double)(global_ns() - t0) > timeout_ns) {
@@ -64,6 +67,11 @@ __device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_n
     }
     __syncthreads();
     return s_err == 0;
+}
+
+// The same over the whole grid, on the launch's own words.
+__device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_ns) {
+    return grid_barrier(c, gen, timeout_ns, &c->bar_count, &c->bar_gen, gridDim.x);
 }
 
 // Start of a tile: thread 0 of each block reads the host's cancel request
@@ -163,7 +171,7 @@ __device__ inline void tile_query_sums(const TravParams &p, long long tile, int 
         }
         if (j == 0) {
             p.tile_partial[tile * 64 + q] = sum;
-            if (flagged) p.qflags[q] |= 1u;
+            if (flagged) atomicOr(&p.qflags[q], 1u);
         }
     }
 }

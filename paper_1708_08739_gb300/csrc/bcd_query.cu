@@ -187,11 +187,12 @@ static bc_status alloc_history(bc_graph *g, int64_t hcap, int64_t ccap, int64_t 
     ws.hcap = hcap;
     ws.ccap = ccap;
     ws.pcap = pcap;
-    BCD_TRY(dev_alloc(&ws.hv, (size_t)hcap));
-    BCD_TRY(dev_alloc(&ws.hm, wg ? (size_t)hmcap : (size_t)hcap * ws.W));
+    const size_t t = (size_t)ws.teams;
+    BCD_TRY(dev_alloc(&ws.hv, t * hcap));
+    BCD_TRY(dev_alloc(&ws.hm, wg ? (size_t)hmcap : t * hcap * ws.W));
     BCD_TRY(dev_alloc(&ws.hs, wg ? (size_t)hcap : (size_t)1));
-    BCD_TRY(dev_alloc(&ws.chunks, (size_t)ccap));
-    BCD_TRY(dev_alloc(&ws.ichunks, wg ? (size_t)1 : (size_t)ccap));
+    BCD_TRY(dev_alloc(&ws.chunks, t * ccap));
+    BCD_TRY(dev_alloc(&ws.ichunks, wg ? (size_t)1 : t * ccap));
     BCD_TRY(dev_alloc(&ws.partial, wg ? (size_t)pcap : (size_t)1));
     BCD_TRY(dev_alloc(&ws.pdone, wg ? (size_t)pcap : (size_t)1));
     BCD_CUDA(cudaMemsetAsync(ws.pdone, 0, sizeof(int32_t) * (size_t)(wg ? pcap : 1), g->stream));
@@ -210,7 +211,7 @@ bc_status alloc_levels(bc_graph *g, int64_t maxlev) {
     dev_free(ws.lev_icstart);
     dev_free(ws.lev_dist);
     ws.maxlev = (int32_t)maxlev;
-    const size_t L = (size_t)maxlev + 2;
+    const size_t L = ((size_t)maxlev + 2) * (size_t)ws.teams;
     BCD_TRY(dev_alloc(&ws.lev_cnt, L));
     BCD_TRY(dev_alloc(&ws.lev_ccnt, L));
     BCD_TRY(dev_alloc(&ws.lev_grab, 6 * L));
@@ -326,6 +327,7 @@ void free_workspace(bc_graph *g) {
     bcd_workspace &ws = g->ws;
     g->root_cache.clear();  // the traversal tables go with the workspace
     g->root_cache_buf = nullptr;
+    dev_free(ws.bar);
     dev_free(ws.vs);
     dev_free(ws.tag);
     dev_free(ws.sigma);
@@ -393,6 +395,30 @@ bc_status ensure_workspace(bc_graph *g, int W) {
     return st;
 }
 
+// Tiles of an unweighted graph that run at once, each by a team of blocks on
+// state of its own. A phase of a level is a chain of about ten dependent loads
+// and a barrier (5-8 us), which a small tile does not fill: on R-MAT 16 (exact
+// batch, 131 tiles) 1 / 2 / 4 / 8 / 16 / 32 teams took 192 / 130 / 107 / 96 /
+// 88 / 94 ms, on 2,000 vertices (8 tiles) 8.9 / 5.4 / 3.4 / 2.4 ms for 1 / 2 /
+// 4 / 8. The larger the tile's state, the less is left to overlap and the more
+// the teams push each other's rows out of L2: R-MAT 18 (7 tiles) 11.5 / 9.0 /
+// 8.8 / 7.9 ms, R-MAT 20 (28 tiles) 356 / 323 / 327 ms for 1 / 2 / 4, R-MAT 22
+// 289 / 280 / 298 ms. All within an eighth of the free memory.
+static int teams_for(int64_t n, int64_t m, int W) {
+    const int64_t rows = n * W / 4;  // vertices in units of a 256-source tile's rows
+    int t = rows <= (1 << 17) ? 16 : rows <= (1 << 19) ? 4 : rows <= (1 << 23) ? 2 : 1;
+    t = (int)std::min<int64_t>(t, std::max<int64_t>(1, (n + 64 * W - 1) / (64 * W)));  // no more than tiles
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    // counts and accumulators 12 S (16 S in fp64), masks and history, chunk lists, level arrays
+    const double per = (double)n * (1024.0 * W + 96.0 * W + 800.0) + 4.0 * (double)m;
+    while (t > 1 && per * t > (double)fr / 8) t >>= 1;
+    return t;
+}
+
 static bc_status build_workspace(bc_graph *g, int W) {
     bcd_workspace &ws = g->ws;
     free_workspace(g);
@@ -402,10 +428,15 @@ static bc_status build_workspace(bc_graph *g, int W) {
     ws.m = m;
     // the weighted kernel keeps no masks; the one-word reach traversals do
     ws.vs_stride = g->weighted ? 4 : ((3 * W + 3) / 4) * 4;
-    BCD_TRY(dev_alloc(&ws.vs, (size_t)n * ws.vs_stride));
-    BCD_TRY(dev_alloc(&ws.tag, (size_t)n));
-    BCD_TRY(dev_alloc(&ws.sigma, (size_t)n * 64 * W));
-    BCD_TRY(dev_alloc(&ws.acc, g->weighted ? (size_t)1 : (size_t)n * 64 * W));
+    ws.teams = g->weighted ? 1 : teams_for(n, m, W);
+    const size_t t = (size_t)ws.teams;
+    BCD_TRY(dev_alloc(&ws.bar, t));
+    BCD_TRY(dev_alloc(&ws.vs, t * n * ws.vs_stride));
+    BCD_TRY(dev_alloc(&ws.tag, t * n));
+    // counts of unweighted graphs: 32 bits until a launch needs fp64; the
+    // accumulators of Eq. 4 come with the first launch that needs them
+    ws.sigma_bytes = g->weighted ? sizeof(double) : sizeof(uint32_t);
+    BCD_TRY(dev_alloc(&ws.sigma, t * n * 64 * W * ws.sigma_bytes / sizeof(double)));
     const int64_t ch = g->chunk_arcs;
     BCD_TRY(alloc_history(g, 8 * n + 4096, 8 * n + 8 * (m / ch) + 4096, 8 * (m / ch) + 4096, 16 * n + 4096));
     BCD_TRY(alloc_levels(g, std::min<int64_t>(g->weighted ? std::max<int64_t>(n + 1, 65536) : n + 1,
@@ -417,19 +448,19 @@ static bc_status build_workspace(bc_graph *g, int W) {
     BCD_TRY(dev_alloc(&ws.hublev, (size_t)n));
     ws.hub = -1;
     BCD_TRY(dev_alloc(&ws.dlist, (size_t)n + 64 * (size_t)W + 256));  // union padded to whole tiles
-    BCD_TRY(dev_alloc(&ws.qlevel, (size_t)64 * W * 64));
-    BCD_TRY(dev_alloc(&ws.dep, (size_t)64 * W * 64));
+    BCD_TRY(dev_alloc(&ws.qlevel, t * 64 * W * 64));
+    BCD_TRY(dev_alloc(&ws.dep, t * 64 * W * 64));
     // vertex scan state
     if (g->weighted)
         BCD_TRY(dev_alloc(&ws.rdist, (size_t)n));
     else
         BCD_TRY(dev_alloc(&ws.rlev, (size_t)n));
     BCD_TRY(dev_alloc(&ws.rsig, (size_t)n));
-    BCD_TRY(dev_alloc(&ws.vsum, (size_t)2 * 64 * W));
-    BCD_TRY(dev_alloc(&ws.msum, (size_t)2 * 64 * W * 64));
+    BCD_TRY(dev_alloc(&ws.vsum, t * 2 * 64 * W));
+    BCD_TRY(dev_alloc(&ws.msum, t * 2 * 64 * W * 64));
     BCD_TRY(dev_alloc(&ws.rtile, (size_t)64 * W));
     BCD_TRY(dev_alloc(&ws.qflags, 64));
-    BCD_TRY(dev_alloc(&ws.srcflag, (size_t)std::max(W, 4)));
+    BCD_TRY(dev_alloc(&ws.srcflag, t * std::max(W, 4)));
     BCD_TRY(dev_alloc(&ws.ctr, 1));
     ws.scratch_len = scan_scratch_len(n) + 64;
     BCD_TRY(dev_alloc(&ws.scratch64, (size_t)ws.scratch_len + 256));
@@ -438,7 +469,7 @@ static bc_status build_workspace(bc_graph *g, int W) {
     BCD_CUDA(cudaMemsetAsync(ws.rvmask, 0, sizeof(uint64_t) * (size_t)n, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.need, 0, sizeof(uint64_t) * (size_t)n, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.qmask, 0, sizeof(uint64_t) * (size_t)n, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.dep, 0, sizeof(double) * 64 * W * 64, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.dep, 0, sizeof(double) * t * 64 * W * 64, g->stream));
     BCD_CUDA(cudaMallocHost(&ws.pinned, 1 << 20));
     ws.pinned_cap = 1 << 20;
     return BC_OK;
@@ -1722,10 +1753,14 @@ bc_status bc_spd_probe(bc_graph *g, const int32_t *sources, int32_t nsrc, const 
         } else if (st == BC_OK) {
             // export sigma [v][S] and the level history
             const size_t n = (size_t)g->n;
-            std::vector<double> sg;
-            if (sigma) {
+            std::vector<double> sg;      // fp64 counts
+            std::vector<uint32_t> sg32;  // or 32-bit counts
+            if (sigma && ws.swide) {
                 sg.resize(n * S);
                 cudaMemcpyAsync(sg.data(), ws.sigma, sizeof(double) * n * S, cudaMemcpyDeviceToHost, s);
+            } else if (sigma) {
+                sg32.resize(n * S);
+                cudaMemcpyAsync(sg32.data(), ws.sigma, sizeof(uint32_t) * n * S, cudaMemcpyDeviceToHost, s);
             }
             std::vector<unsigned long long> lc(ws.maxlev + 2);
             cudaMemcpyAsync(lc.data(), ws.lev_cnt, sizeof(unsigned long long) * lc.size(), cudaMemcpyDeviceToHost, s);
@@ -1754,7 +1789,7 @@ bc_status bc_spd_probe(bc_graph *g, const int32_t *sources, int32_t nsrc, const 
                         for (int i = 0; i < nsrc; ++i) {
                             if ((hm[e * W + (i >> 6)] >> (i & 63)) & 1ull) {
                                 if (dist) dist[(size_t)i * n + v] = (uint64_t)L;
-                                if (sigma) sigma[(size_t)i * n + v] = sg[(size_t)v * S + i];
+                                if (sigma) sigma[(size_t)i * n + v] = ws.swide ? sg[(size_t)v * S + i] : (double)sg32[(size_t)v * S + i];
                             }
                         }
                     }

@@ -1,16 +1,24 @@
 // Persistent multi-source traversal: the single-source work of Algorithm 1
 // (and Algorithm 2) for S = 64*W sources at once.
 //
-// One cooperative launch walks every tile of S sources. Per tile:
-//   forward  (Section 2): level-synchronous BFS over the forward CSR, one
-//            grid barrier per level. Per vertex the dense state holds the
-//            visited mask and two level-parity masks (bit s: vertex is at the
-//            current / next level for source s). Frontier vertices are pushed
-//            along their out-arcs in chunks of at most chunk_arcs arcs; for
-//            every arc (u, v) the sources newly reaching v are
-//            F(u) & ~(visited(v) | current(v)), and sigma_s(v) += sigma_s(u)
-//            by an fp64 atomic add (sigma are integers, so the sum is exact
-//            in any order while below 2^53).
+// One cooperative launch walks every tile of S sources. Its blocks form one or
+// more teams, each with the state of one tile and a barrier of its own; a team
+// takes the next tile when it has finished one, so that one tile's thin levels
+// and barriers overlap another's work (bcd_query.cu, teams_for). Per tile:
+//   forward  (Section 2): level-synchronous BFS over the forward CSR. Per
+//            vertex the dense state holds the visited mask (levels up to the
+//            current one) and two level-parity masks (bit s: vertex is at the
+//            current / next level for source s). A level runs in two phases
+//            with a grid barrier after each:
+//              push    (push_masks) the frontier's out-arcs (u, v), in chunks
+//                      of at most chunk_arcs arcs, mark the sources newly
+//                      reaching v, F(u) & ~visited(v), in v's next-level mask;
+//              gather  (gather_level) every vertex of the next level sums
+//                      sigma_s(v) over its in-arcs (R(G)) from the
+//                      in-neighbours on the current level, in registers, and
+//                      writes its sigma row once.
+//            Sigma are integers, exact in any order: held as 32-bit counts, or
+//            as fp64 after a launch met a count of 2^26 (it reruns).
 //   backward (Eq. 4): levels from the deepest one up to the shallowest level
 //            any query vertex sits at. With c_s(w) = (1 + delta_s(w)) /
 //            sigma_s(w), delta_s(v) = sigma_s(v) * sum over tight out-arcs
@@ -44,19 +52,154 @@ namespace {
 
 using namespace dev;
 
-// Appends the vertices a warp discovered at level L+1: one entry and its
-// out-arc chunks each and, in SPD mode, the in-arc (R(G)) chunks the backward
-// pass pushes along, with one set of counter atomics per warp.
+// Per-thread work counters (flushed to the 64-bit launch totals at the end of
+// every tile).
+struct Stats {
+    unsigned long long edges = 0;
+    unsigned reached = 0, tight = 0, arcs = 0;
+};
+
+__device__ __forceinline__ void flush_stats(Counters *c, Stats &st, int lane) {
+    unsigned long long v[4] = {st.edges, st.reached, st.tight, st.arcs};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(kFull, v[i], o);
+    if (lane == 0) {
+        unsigned long long *dst[4] = {&c->edges, &c->reached, &c->tight, &c->arc_visits};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (v[i]) atomicAdd(dst[i], v[i]);
+    }
+    st = Stats();
+}
+
+// Path counts: 32-bit integers are trusted below 2^26, so that a sum of 33
+// terms cannot wrap before it is tested; fp64 sums need no such test.
+constexpr uint32_t kCountLimit = 1u << 26;
+
+template <typename T>
+struct SigOver {
+    static __device__ __forceinline__ unsigned test(T x) { return 0u; }
+};
+template <>
+struct SigOver<uint32_t> {
+    static __device__ __forceinline__ unsigned test(uint32_t x) { return x & ~(kCountLimit - 1u); }
+};
+
+// Source s met a count of 2^53 (fp64 counts only).
+__device__ __forceinline__ void flag_two53(const TravParams &p, uint32_t, int) {}
+__device__ __forceinline__ void flag_two53(const TravParams &p, double x, int s) {
+    if (x >= 9007199254740992.0) atomicOr((unsigned long long *)&p.srcflag[s >> 6], 1ull << (s & 63));
+}
+
+// Where the next level's entries and chunks start in the history.
+struct LevelEnds {
+    long long es, cs, ics;
+};
+
+// Per-warp staging of the packed chunk groups of push_masks and gather_level.
+constexpr int kGroup = 8;  // chunks a warp takes together
+template <int W>
+struct __align__(16) WarpBuf {
+    uint64_t n[kGroup][W];   // source masks of the group's entries
+    uint64_t t[32][W];       // gather: tight sources of the 32 arcs in hand
+    long long aoff[kGroup];  // arc i of the group sits at aoff[chunk] + i
+    int incl[kGroup];        // arcs of the group up to and with each chunk
+    int v[kGroup];           // gather: the entries' vertices
+    int nch[kGroup];         // gather: in-arc chunks of the vertex
+    struct {                 // the phase's chunk hand-out (GroupGrabber)
+        unsigned long long *ctr;
+        long long cnt, first;
+        int grab;
+    } hand;
+    long long first;         // first chunk of the level in hand
+    LevelEnds ends;          // ... and where its successors go
+    Stats st[32];            // work counters of the warp's lanes
+    unsigned q[128];         // vertices claimed for the next level, not yet appended (kFirstSeen: new to the tile)
+
+    // Stages lane i's chunk (na arcs from a0) and returns the group's arcs.
+    __device__ __forceinline__ int pack(int lane, int na, long long a0) {
+        int x = na;
+#pragma unroll
+        for (int o = 1; o < kGroup; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane < kGroup) {
+            incl[lane] = x;
+            aoff[lane] = a0 - (x - na);
+        }
+        __syncwarp();
+        return incl[kGroup - 1];
+    }
+
+    // The chunk that holds arc i of the group.
+    __device__ __forceinline__ int find(int i) const {
+        int j = 0;
+#pragma unroll
+        for (int o = kGroup / 2; o > 0; o >>= 1)
+            if (incl[j + o - 1] <= i) j += o;
+        return j;
+    }
+};
+
+constexpr unsigned kFirstSeen = 0x80000000u;
+
+// Dynamic shared memory: the launch's parameters, the queries each source
+// slot of the tile serves (64 W words), then one WarpBuf per warp (or a
+// ScanBuf). The functions that are not inlined take these from here, not as
+// arguments: a reference argument would turn every access, also to the
+// parameters, into a generic load.
+extern __shared__ __align__(16) unsigned char s_dyn[];
+constexpr int kParamBytes = ((int)sizeof(TravParams) + 15) / 16 * 16;
+__device__ __forceinline__ const TravParams &shared_params() { return *reinterpret_cast<const TravParams *>(s_dyn); }
+__device__ __forceinline__ uint64_t *tile_need() { return reinterpret_cast<uint64_t *>(s_dyn + kParamBytes); }
+template <int W>
+__device__ __forceinline__ WarpBuf<W> &warp_buf() {
+    return reinterpret_cast<WarpBuf<W> *>(s_dyn + kParamBytes + 512 * W)[threadIdx.x >> 5];
+}
+
+// Appends the first `take` (at most 32) of a warp's claimed vertices to level
+// L + 1, one per lane: one entry and its out-arc chunks each and, unless only
+// reach is asked, the in-arc (R(G)) chunks that the gather (and the Eq. 4
+// backward) walks, with one set of counter atomics per warp. The out-degree
+// rides in the chunks. Claims are queued per warp and appended 32 at a time,
+// so that the atomics' round trip is paid once per 32 vertices.
 template <int W, int MODE>
-__device__ __forceinline__ void warp_append(const TravParams &p, int L, bool app, int wv, int wnch, long long wrb,
-                                            long long wre, int winch, long long wirb, long long wire, long long es1,
-                                            long long cs1, long long ics1, int lane) {
-    const unsigned am = __ballot_sync(kFull, app);
-    if (am == 0) return;
-    const int rank = __popc(am & ((1u << lane) - 1u));
-    const int ne = __popc(am);
-    int x = app ? wnch : 0;
-    int xi = app ? winch : 0;
+__device__ __noinline__ void append_queue(int L, int qn, int take) {
+    const TravParams &p = shared_params();
+    WarpBuf<W> &buf = warp_buf<W>();
+    const LevelEnds &ends = buf.ends;
+    const int lane = threadIdx.x & 31;
+    const int CH = p.chunk_arcs;
+    const bool app = lane < take;
+    int wv = 0, wnch = 0, winch = 0;
+    long long wrb = 0, wirb = 0;
+    int deg = 0, ideg = 0;
+    unsigned vb = 0;
+    __syncwarp();
+    if (app) {
+        const unsigned x = buf.q[lane];
+        wv = (int)(x & ~kFirstSeen);
+        vb = x >> 31;
+        wrb = p.off[wv];
+        deg = (int)(p.off[wv + 1] - wrb);
+        wnch = max(1, (deg + CH - 1) / CH);
+        if (MODE != kModeReach) {
+            wirb = p.roff[wv];
+            ideg = (int)(p.roff[wv + 1] - wirb);
+            winch = (ideg + CH - 1) / CH;
+        }
+    }
+    // the rest of the queue moves to its front
+    unsigned rest[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) rest[k] = 32 * (k + 1) + lane < qn ? buf.q[32 * (k + 1) + lane] : 0u;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) buf.q[32 * k + lane] = rest[k];
+    int x = wnch, xi = winch;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(kFull, x, o);
@@ -66,46 +209,150 @@ __device__ __forceinline__ void warp_append(const TravParams &p, int L, bool app
             xi += yi;
         }
     }
-    const int tot = __shfl_sync(kFull, x, 31);
-    const int toti = __shfl_sync(kFull, xi, 31);
     // out-arcs of the appended vertices: the next level's frontier arcs, which
-    // choose its direction
-    unsigned long long fa = app ? (unsigned long long)(wre - wrb) : 0ull;
+    // choose its direction; and of those, the ones new to the tile
+    unsigned long long fa = (unsigned long long)deg, fb = vb ? (unsigned long long)deg : 0ull;
+    if (MODE != kModeReach) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) fa += __shfl_xor_sync(kFull, fa, o);
-    unsigned long long eb = 0, cb = 0, ib = 0;
-    if (lane == 0) {
+        for (int o = 16; o > 0; o >>= 1) {
+            fa += __shfl_xor_sync(kFull, fa, o);
+            fb += __shfl_xor_sync(kFull, fb, o);
+        }
+        vb = __popc(__ballot_sync(kFull, vb != 0u));
+    }
+    const long long nl = (long long)p.maxlev + 2;
+    unsigned long long old = 0, ib = 0;
+    if (lane == 31) {
         // entries (low half) and out-arc chunks (high half) in one atomic: every
         // appending warp of the level meets on this word
-        const unsigned long long old =
-            atomicAdd(&p.lev_grab[4 * ((long long)p.maxlev + 2) + L + 1], (unsigned long long)ne | ((unsigned long long)tot << 32));
-        eb = old & 0xffffffffull;
-        cb = old >> 32;
-        if (MODE == kModeSpd && toti)
-            ib = atomicAdd(&p.lev_grab[2 * ((long long)p.maxlev + 2) + L + 1], (unsigned long long)toti);
-        if (MODE != kModeReach && fa && p.pull_arcs_min > 0)
-            atomicAdd(&p.lev_grab[3 * ((long long)p.maxlev + 2) + L + 1], fa);
+        old = atomicAdd(&p.lev_grab[4 * nl + L + 1], (unsigned long long)take | ((unsigned long long)x << 32));
+        if (MODE != kModeReach) {
+            if (xi) ib = atomicAdd(&p.lev_grab[2 * nl + L + 1], (unsigned long long)xi);
+            if (fa && p.pull_arcs_min > 0) atomicAdd(&p.lev_grab[3 * nl + L + 1], fa);
+            if (vb) atomicAdd(&p.ctr->vb, (unsigned long long)vb);
+            if (fb) atomicAdd(&p.ctr->eb, fb);
+        }
     }
-    eb = __shfl_sync(kFull, eb, 0);
-    cb = __shfl_sync(kFull, cb, 0);
-    if (MODE == kModeSpd) ib = __shfl_sync(kFull, ib, 0);
+    old = __shfl_sync(kFull, old, 31);
+    if (MODE != kModeReach) ib = __shfl_sync(kFull, ib, 31);
     if (app) {
-        const long long e = es1 + (long long)eb + rank;
-        const long long c0 = cs1 + (long long)cb + (x - wnch);
-        const long long i0 = ics1 + (long long)ib + (xi - winch);
+        const long long e = ends.es + (long long)(old & 0xffffffffull) + lane;
+        const long long c0 = ends.cs + (long long)(old >> 32) + (x - wnch);
+        const long long i0 = ends.ics + (long long)ib + (xi - winch);
         if (e >= p.hcap) {
             set_err(p.ctr, kDevHistOverflow);
-        } else if (c0 + wnch > p.ccap || (MODE == kModeSpd && i0 + winch > p.ccap)) {
+        } else if (c0 + wnch > p.ccap || (MODE != kModeReach && i0 + winch > p.ccap)) {
             set_err(p.ctr, kDevChunkOverflow);
         } else {
             p.hv[e] = wv;
-            emit_chunks(p, c0, wv, (int)e, wnch, wrb, wre);
-            if (MODE == kModeSpd) {
-                const int CH = p.chunk_arcs;
-                for (int k = 0; k < winch; ++k) {
-                    const long long a0 = wirb + (long long)k * CH;
-                    store_chunk(&p.ichunks[i0 + k], wv, (int)e, k, winch, a0, (int)(min(wire, a0 + CH) - a0));
-                }
+            emit_chunks(p, c0, wv, (int)e, wnch, wrb, wrb + deg);
+            if (MODE != kModeReach)
+                for (int k = 0; k < winch; ++k)
+                    store_chunk(&p.ichunks[i0 + k], wv, (int)e, k, winch, wirb + (long long)k * CH,
+                                min(CH, ideg - k * CH), deg);
+        }
+    }
+    __syncwarp();
+}
+
+// Queues the vertices that lanes with `app` claimed.
+template <int W>
+__device__ __forceinline__ void claim(WarpBuf<W> &buf, int &qn, bool app, unsigned x, int lane) {
+    const unsigned am = __ballot_sync(kFull, app);
+    if (app) buf.q[qn + __popc(am & ((1u << lane) - 1u))] = x;
+    qn += __popc(am);
+}
+
+// Appends whole warps of the queue (all of it at the end of a level).
+template <int W, int MODE>
+__device__ __forceinline__ void drain(int L, int &qn, bool all) {
+    while (qn >= 32 || (all && qn > 0)) {
+        const int take = min(qn, 32);
+        append_queue<W, MODE>(L, qn, take);
+        qn -= take;
+    }
+}
+
+// The W words of a mask (16-byte loads where the row allows them).
+template <int W>
+__device__ __forceinline__ void load_mask(const uint64_t *row, uint64_t (&m)[W]) {
+    if (W == 1) {
+        m[0] = row[0];
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; w += 2) {
+            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(row + w);
+            m[w] = x.x;
+            m[W > 1 ? w + 1 : 0] = x.y;
+        }
+    }
+}
+
+// Hand-out of a level's chunks in groups of up to kGroup consecutive ones
+// (fewer when the level is thin, so that all warps get some). The first group
+// of each warp is fixed and the rest are drawn from a counter: on a thin level
+// no warp touches the counter, where all warps of the grid would queue up.
+template <int W>
+struct GroupGrabber {
+    long long at;
+    __device__ GroupGrabber(unsigned long long *c, long long n, long long gwarp, long long nwarps) {
+        WarpBuf<W> &buf = warp_buf<W>();
+        const long long g = max(1ll, min((long long)kGroup, n / (nwarps * 4)));
+        at = gwarp * g;
+        __syncwarp();
+        buf.hand.ctr = c;
+        buf.hand.cnt = n;
+        buf.hand.first = nwarps * g;
+        buf.hand.grab = (int)g;
+        __syncwarp();
+    }
+    // The next group: its size (0: none left) and, in c0, its first chunk.
+    __device__ __forceinline__ int next(long long &c0, int lane) {
+        const auto &h = warp_buf<W>().hand;
+        const long long cnt = h.cnt;
+        if (at >= cnt) return 0;
+        c0 = at;
+        const int k = (int)min((long long)h.grab, cnt - at);
+        at = cnt;
+        if (h.first < cnt) {
+            unsigned long long b = 0;
+            if (lane == 0) b = atomicAdd(h.ctr, (unsigned long long)h.grab);
+            at = h.first + (long long)__shfl_sync(kFull, b, 0);
+        }
+        return k;
+    }
+};
+
+// The bookkeeping of an entry (v, F) that joins level L (one thread): its
+// mask into the history and the visited set, the work counters, and the level
+// of the query vertices that sit at v.
+template <int W>
+__device__ __forceinline__ void enter_entry(const TravParams &p, int L, long long e, int v, const uint64_t (&F)[W],
+                                            const uint64_t (&vis)[W], int odeg, Stats &st) {
+    const uint64_t *s_need = tile_need();
+    uint64_t *row = p.vs + (size_t)v * p.vs_stride;
+    int pc = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        p.hm[(size_t)e * W + w] = F[w];
+        row[w] = vis[w] | F[w];
+        pc += __popcll(F[w]);
+    }
+    st.edges += (unsigned long long)pc * (unsigned)odeg;
+    st.reached += (unsigned)pc;
+    const uint64_t qm = p.qmask[v];
+    if (qm == 0ull) return;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        uint64_t b = F[w];
+        while (b) {
+            const int s = 64 * w + __ffsll((long long)b) - 1;
+            b &= b - 1;
+            uint64_t x = qm & s_need[s];
+            while (x) {
+                const int q = __ffsll((long long)x) - 1;
+                x &= x - 1;
+                p.qlevel[s * 64 + q] = L;
             }
         }
     }
@@ -113,7 +360,7 @@ __device__ __forceinline__ void warp_append(const TravParams &p, int L, bool app
 
 // Level 0 of a tile: one entry per source slot (block 0 only). Thread t
 // seeds slot t: the launch has at least S threads per block.
-template <int W, int MODE>
+template <int W, int MODE, typename T>
 __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
     constexpr int S = 64 * W;
     __shared__ int s_scan[S];
@@ -131,6 +378,13 @@ __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
         s_scan[t] = nch;
     }
     if (t == 0) s_valid = 0;
+    if (MODE != kModeReach) {
+        for (int i = t; i < S * 64; i += blockDim.x) p.qlevel[i] = -1;
+        if (t < W) p.srcflag[t] = 0ull;
+    }
+    if (MODE == kModeScan && t < S) p.vsum[t] = 0.0;
+    if (MODE == kModeScan && p.ncols >= 2)
+        for (int i = t; i < S * 64; i += blockDim.x) p.msum[i] = 0.0;
     __syncthreads();
     if (t < S && v >= 0) atomicAdd(&s_valid, 1);
     for (int o = 1; o < S; o <<= 1) {
@@ -150,7 +404,8 @@ __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
             for (int w = 0; w < W; ++w) {
                 const uint64_t b = (w == (t >> 6)) ? (1ull << (t & 63)) : 0ull;
                 p.hm[(size_t)t * W + w] = b;
-                row[W + w] = b;  // level-0 parity mask
+                row[W + w] = b;                       // level-0 parity mask
+                if (MODE != kModeReach) row[w] = b;   // visited (the reach push sets it itself)
             }
             p.hv[t] = v;
             p.tag[v] = 0;
@@ -158,17 +413,18 @@ __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
             if (MODE != kModeReach) {
                 atomicAdd(&p.ctr->vb, 1ull);
                 atomicAdd(&p.ctr->eb, (unsigned long long)(re - rb));
+                atomicAdd(&p.ctr->edges, (unsigned long long)(re - rb));
+                atomicAdd(&p.ctr->reached, 1ull);
+                reinterpret_cast<T *>(p.sigma)[(size_t)v * S + t] = T(1);
+                uint64_t x = p.qmask[v] & p.need[v];
+                while (x) {
+                    const int q = __ffsll((long long)x) - 1;
+                    x &= x - 1;
+                    p.qlevel[t * 64 + q] = 0;
+                }
             }
-            if (MODE != kModeReach) p.sigma[(size_t)v * S + t] = 1.0;
         }
     }
-    if (MODE != kModeReach) {
-        for (int i = t; i < S * 64; i += blockDim.x) p.qlevel[i] = -1;
-        if (t < W) p.srcflag[t] = 0ull;
-    }
-    if (MODE == kModeScan && t < S) p.vsum[t] = 0.0;
-    if (MODE == kModeScan && p.ncols >= 2)
-        for (int i = t; i < S * 64; i += blockDim.x) p.msum[i] = 0.0;
     __syncthreads();
     if (t == 0) {
         p.lev_cnt[0] = (unsigned long long)s_valid;
@@ -177,264 +433,289 @@ __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
     }
 }
 
-// Expansion of level L (forward pass, Section 2 / Section 4.1). Lane l holds
-// sources l + 32 i; the next 32 heads are fetched while the current ones'
-// masks are read.
-// Per-thread work counters (32-bit; flushed to the 64-bit launch totals at
-// the end of every tile).
-struct Stats {
-    unsigned edges = 0, reached = 0, tight = 0, arcs = 0, vb = 0, eb = 0;
-};
-
-__device__ __forceinline__ void flush_stats(Counters *c, Stats &st, int lane) {
-    unsigned long long v[6] = {st.edges, st.reached, st.tight, st.arcs, st.vb, st.eb};
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(kFull, v[i], o);
-    if (lane == 0) {
-        unsigned long long *dst[6] = {&c->edges, &c->reached, &c->tight, &c->arc_visits, &c->vb, &c->eb};
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-            if (v[i]) atomicAdd(dst[i], v[i]);
-    }
-    st = Stats();
-}
-
-// Expansion of one out-arc chunk of a level-L entry (forward pass): the
-// descriptor, the frontier mask F of its vertex and this lane's first head
-// come in loaded, so the caller can fetch them ahead of time.
-template <int W, int MODE>
-__device__ __forceinline__ void expand_chunk(const TravParams &p, int L, const Chunk &ch, const uint64_t (&F)[W],
-                                             int wv_next, long long es1, long long cs1, long long ics1, Stats &st,
-                                             const uint64_t *s_need) {
-    constexpr int S = 64 * W;
-    constexpr int PL = 2 * W;
+// Push phase of level L: the frontier's out-arcs (u, v) mark F(u) &
+// ~visited(v) in v's next-level mask; a vertex marked first at this level is
+// claimed (an atomic on its level tag) and appended. A warp takes up to kGroup
+// consecutive chunks and packs their arcs onto its lanes (two arcs per lane in
+// flight), so short rows do not leave lanes idle; an arc costs its head and
+// one W-word mask. The next-level mask is read before it is changed: most arcs
+// into a hub find their bits set already, and the same-address atomics that
+// would follow were what the hubs' rows waited for. Reach mode keeps one
+// barrier per level, so it excludes the current level's mask too and does the
+// entries' bookkeeping here.
+template <int W, int MODE, int U>
+__device__ __noinline__ void push_masks(int L, long long ccnt, long long gwarp, long long nwarps) {
+    const TravParams &p = shared_params();
+    WarpBuf<W> &buf = warp_buf<W>();
     const int lane = threadIdx.x & 31;
     const int cur = 1 + (L & 1);
     const int nxt = 1 + ((L + 1) & 1);
-    const int stride = p.vs_stride;
-    const int CH = p.chunk_arcs;
-    const int v = ch.v, e = ch.e;
-    const long long a0 = ch.a0;
-    const int na = ch.na;
-    double sig[PL];
-    if (MODE != kModeReach) {
-        // only the frontier's sources: sectors of the row without one are not read
+    int qn = 0;  // claimed vertices in the queue
+    GroupGrabber<W> grab(&p.lev_grab[L], ccnt, gwarp, nwarps);
+    for (;;) {
+        long long c0;
+        const int cnt = grab.next(c0, lane);
+        if (cnt == 0) break;
+        int na = 0;
+        long long a0 = 0;
+        if (lane < cnt) {
+            const Chunk ch = load_chunk(&p.chunks[buf.first + c0 + lane]);
+            na = ch.na;
+            a0 = ch.a0;
+            uint64_t F[W];
+            if (MODE == kModeReach)
+                load_mask<W>(p.vs + (size_t)ch.v * p.vs_stride + cur * W, F);
+            else
+                load_mask<W>(p.hm + (size_t)ch.e * W, F);
 #pragma unroll
-        for (int ii = 0; ii < PL; ++ii)
-            sig[ii] = mask_bit<W>(F, lane + 32 * ii) ? p.sigma[(size_t)v * S + lane + 32 * ii] : 0.0;
-    }
-    if (ch.k == 0) {
-        if (MODE == kModeReach && p.levout && lane == 0 && p.levout[v] < 0) p.levout[v] = L;
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-            if (lane == w) p.hm[(size_t)e * W + w] = F[w];
-        // visited |= F: reductions that need no answer (the sources of F are
-        // already excluded from new bits by the current-level mask)
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-            if (lane == w) atomicOr((unsigned long long *)&p.vs[(size_t)v * stride + w], (unsigned long long)F[w]);
-        if (MODE != kModeReach) {
-            if (lane == 0) {
-                int pc = 0;
-#pragma unroll
-                for (int w = 0; w < W; ++w) pc += __popcll(F[w]);
-                st.edges += (unsigned)pc * (unsigned)ch.pad;  // out-degree of v rides in the chunk
-                st.reached += (unsigned)pc;
-            }
-            const uint64_t qm = p.qmask[v];
-#pragma unroll
-            for (int ii = 0; ii < PL; ++ii) {
-                const int s = lane + 32 * ii;
-                if (mask_bit<W>(F, s)) {
-                    if (qm) {
-                        uint64_t x = qm & s_need[s];
-                        while (x) {
-                            const int q = __ffsll((long long)x) - 1;
-                            x &= x - 1;
-                            p.qlevel[s * 64 + q] = L;
-                        }
-                    }
-                    if (sig[ii] >= 9007199254740992.0)
-                        atomicOr((unsigned long long *)&p.srcflag[s >> 6], 1ull << (s & 63));
-                }
-            }
-        }
-    }
-    for (int base = 0; base < na; base += 32) {
-        const bool valid = base + lane < na;
-        const int wv = wv_next;
-        wv_next = base + 32 + lane < na ? p.col[a0 + base + 32 + lane] : 0;
-        uint64_t nm[W];
-        bool any = false;
-        if (valid) {
-            const uint64_t *wrow = p.vs + (size_t)wv * stride;
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                nm[w] = F[w] & ~(wrow[w] | wrow[cur * W + w]);
-                any |= nm[w] != 0ull;
-            }
-            if (MODE != kModeReach) {
-                st.arcs += 1;
-#pragma unroll
-                for (int w = 0; w < W; ++w) st.tight += (unsigned)__popcll(nm[w]);
-            }
-        } else {
-#pragma unroll
-            for (int w = 0; w < W; ++w) nm[w] = 0ull;
-        }
-        // heads with new sources: mark them for the next level and claim
-        // the level's entry; the claim's answer (and the row bounds) are
-        // used only after the sigma adds, so their round trips overlap
-        int old = 0x7fffffff;
-        long long wrb = 0, wre = 0, wirb = 0, wire = 0;
-        if (any) {
-            uint64_t *wrow = p.vs + (size_t)wv * stride;
-#pragma unroll
-            for (int w = 0; w < W; ++w)
-                if (nm[w]) atomicOr((unsigned long long *)&wrow[nxt * W + w], (unsigned long long)nm[w]);
-            old = atomicMax(&p.tag[wv], L + 1);
-            wrb = p.off[wv];
-            wre = p.off[wv + 1];
-            if (MODE == kModeSpd) {
-                wirb = p.roff[wv];
-                wire = p.roff[wv + 1];
-            }
-        }
-        if (MODE != kModeReach) {
-            // two tight heads per step: their shuffles and atomics overlap
-            unsigned bal = __ballot_sync(kFull, any);
-            while (bal) {
-                const int i0 = __ffs(bal) - 1;
-                bal &= bal - 1;
-                const int i1 = bal ? __ffs(bal) - 1 : -1;
-                if (bal) bal &= bal - 1;
-                const int j1 = i1 < 0 ? i0 : i1;
-                const int w0 = __shfl_sync(kFull, wv, i0);
-                const int w1 = __shfl_sync(kFull, wv, j1);
-                uint64_t n0[W], n1[W];
+            for (int w = 0; w < W; ++w) buf.n[lane][w] = F[w];
+            if (MODE == kModeReach && ch.k == 0) {
+                if (p.levout && p.levout[ch.v] < 0) p.levout[ch.v] = L;
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
-                    n0[w] = __shfl_sync(kFull, nm[w], i0);
-                    n1[w] = __shfl_sync(kFull, nm[w], j1);
-                }
-                if (i1 < 0) {
-#pragma unroll
-                    for (int w = 0; w < W; ++w) n1[w] = 0ull;
-                }
-                double *r0 = p.sigma + (size_t)w0 * S;
-                double *r1 = p.sigma + (size_t)w1 * S;
-#pragma unroll
-                for (int ii = 0; ii < PL; ++ii) {
-                    const int s = lane + 32 * ii;
-                    if (mask_bit<W>(n0, s)) atomicAdd(&r0[s], sig[ii]);
-                    if (mask_bit<W>(n1, s)) atomicAdd(&r1[s], sig[ii]);
+                    p.hm[(size_t)ch.e * W + w] = F[w];
+                    atomicOr((unsigned long long *)&p.vs[(size_t)ch.v * p.vs_stride + w], (unsigned long long)F[w]);
                 }
             }
         }
-        const bool app = any && old < L + 1;
-        int wnch = 0, winch = 0;
-        if (app) {
-            wnch = (int)max(1ll, (wre - wrb + CH - 1) / CH);
-            if (MODE == kModeSpd) winch = (int)((wire - wirb + CH - 1) / CH);
-            if (MODE != kModeReach && old < 0) {
-                st.vb += 1;
-                st.eb += (unsigned)(wre - wrb);
-            }
+        const int total = buf.pack(lane, na, a0);
+        if (MODE != kModeReach && lane == 0) buf.st[0].arcs += (unsigned)total;
+        int base = 0;
+        while (base < total) {
+            // arcs until the queue holds more than it could take of another step's claims
+            int wn[U], jn[U];
+            auto fetch = [&](int b) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = b + 32 * u + lane;
+                    jn[u] = buf.find(i);
+                    wn[u] = i < total ? __ldcs(p.col + buf.aoff[jn[u]] + i) : -1;
+                }
+            };
+            fetch(base);
+            do {
+                int wv[U], j[U];
+                uint64_t nm[U][W];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    wv[u] = wn[u];
+                    j[u] = jn[u];
+                    if (wv[u] >= 0) {
+                        load_mask<W>(p.vs + (size_t)wv[u] * p.vs_stride, nm[u]);
+                        if (MODE == kModeReach) {
+                            uint64_t c[W];
+                            load_mask<W>(p.vs + (size_t)wv[u] * p.vs_stride + cur * W, c);
+#pragma unroll
+                            for (int w = 0; w < W; ++w) nm[u][w] |= c[w];
+                        }
+                    }
+                }
+                base += 32 * U;
+                fetch(base);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    bool any = false;
+                    if (wv[u] >= 0) {
+#pragma unroll
+                        for (int w = 0; w < W; ++w) {
+                            nm[u][w] = buf.n[j[u]][w] & ~nm[u][w];
+                            any |= nm[u][w] != 0ull;
+                        }
+                    }
+                    int old = 0x7fffffff;
+                    if (any) {
+                        uint64_t *wrow = p.vs + (size_t)wv[u] * p.vs_stride + nxt * W;
+                        const int tg = p.tag[wv[u]];
+                        uint64_t nx[W];
+                        load_mask<W>(wrow, nx);
+                        bool add = false;
+#pragma unroll
+                        for (int w = 0; w < W; ++w) {
+                            const uint64_t x = nm[u][w] & ~nx[w];
+                            if (x) {
+                                atomicOr((unsigned long long *)&wrow[w], (unsigned long long)x);
+                                add = true;
+                            }
+                        }
+                        if (add && tg < L + 1) old = atomicMax(&p.tag[wv[u]], L + 1);
+                    }
+                    claim<W>(buf, qn, old < L + 1, (unsigned)wv[u] | (old < 0 ? kFirstSeen : 0u), lane);
+                }
+            } while (base < total && qn <= 128 - 32 * U);
+            drain<W, MODE>(L, qn, false);
         }
-        warp_append<W, MODE>(p, L, app, wv, wnch, wrb, wre, winch, wirb, wire, es1, cs1, ics1, lane);
+        __syncwarp();
     }
+    drain<W, MODE>(L, qn, true);
 }
 
-// Expansion of level L (forward pass, Section 2 / Section 4.1). A warp takes
-// the level's chunks from the dynamic hand-out. With PIPE (the one-block-per-
-// SM kernels, which have the registers) the loop runs three chunks deep: the
-// descriptor of chunk i + 2 and the frontier mask and first heads of chunk
-// i + 1 are in flight while chunk i expands, so a chunk starts with one round
-// trip (sigma and the heads' masks) instead of three.
-template <int W, int MODE, bool PIPE>
-__device__ void forward_level(const TravParams &p, int L, long long cs, long long ccnt, long long es1,
-                              long long cs1, long long ics1, Stats &st, const uint64_t *s_need,
-                              long long gwarp, long long nwarps) {
+// Gather phase: the vertices v of level L (their masks N(v) complete since
+// the barrier after the push) sum sigma_s(v) = sum over in-neighbours u at
+// level L - 1 for s of sigma_s(u). A warp takes up to kGroup consecutive
+// in-arc chunks and packs their arcs onto its lanes: each lane reads one
+// in-neighbour's level mask, t = current(u) & N(v), and stages it; then the
+// warp walks the arcs with a tight source, U rows in flight, lane l holding
+// sources l + 32 i: one test, one predicated load and one addition per 32
+// sources (the masks are sparse, about a sixth of the tile, so wider loads
+// would spend their instructions on sources that are not there). A row that
+// fits one chunk is written once; longer rows meet in atomic adds on a row
+// that starts from zero.
+template <int W, typename T, int U>
+__device__ __noinline__ void gather_level(int L, long long ics, long long iccnt, long long gwarp, long long nwarps) {
+    const TravParams &p = shared_params();
+    constexpr int S = 64 * W;
+    constexpr int PL = 2 * W;
+    WarpBuf<W> &buf = warp_buf<W>();
     const int lane = threadIdx.x & 31;
-    const int cur = 1 + (L & 1);
-    const int stride = p.vs_stride;
-    ChunkGrabber grab(&p.lev_grab[L], ccnt, nwarps);
-    if (!PIPE) {
-        long long c;
-        while (grab.next(c, lane)) {
-            const Chunk ch = load_chunk(&p.chunks[cs + c]);
-            const int w0 = lane < ch.na ? p.col[ch.a0 + lane] : 0;
-            const uint64_t *vrow = p.vs + (size_t)ch.v * stride;
+    const uint32_t lbit = 1u << lane;
+    const int prv = 1 + ((L - 1) & 1);  // slot of the level-(L - 1) masks (level L: the other one)
+    T *const sigma = reinterpret_cast<T *>(p.sigma) + lane;
+    unsigned over = 0, tight = 0;
+    if (lane == 0) buf.first = ics;
+    T acc[PL];
+#pragma unroll
+    for (int q = 0; q < PL; ++q) acc[q] = T(0);
+    GroupGrabber<W> grab(&p.lev_grab[5 * ((long long)p.maxlev + 2) + L], iccnt, gwarp, nwarps);
+    for (;;) {
+        long long c0;
+        const int cnt = grab.next(c0, lane);
+        if (cnt == 0) break;
+        int na = 0;
+        long long a0 = 0;
+        if (lane < cnt) {
+            const Chunk ch = load_chunk(&p.ichunks[buf.first + c0 + lane]);
+            buf.v[lane] = ch.v;
+            buf.nch[lane] = ch.nch;
+            na = ch.na;
+            a0 = ch.a0;
+            const uint64_t *row = p.vs + (size_t)ch.v * p.vs_stride;
             uint64_t F[W];
+            load_mask<W>(row + (3 - prv) * W, F);
 #pragma unroll
-            for (int w = 0; w < W; ++w) F[w] = vrow[cur * W + w];
-            expand_chunk<W, MODE>(p, L, ch, F, w0, es1, cs1, ics1, st, s_need);
+            for (int w = 0; w < W; ++w) buf.n[lane][w] = F[w];
+            if (ch.k == 0) {
+                uint64_t vis[W];
+                load_mask<W>(row, vis);
+                enter_entry<W>(p, L, ch.e, ch.v, F, vis, ch.pad, buf.st[lane]);
+            }
         }
-        return;
-    }
-    Chunk d0{}, d1{};
-    long long c0 = 0, c1 = 0;
-    bool h0 = grab.next(c0, lane);
-    if (h0) d0 = load_chunk(&p.chunks[cs + c0]);
-    bool h1 = h0 && grab.next(c1, lane);
-    if (h1) d1 = load_chunk(&p.chunks[cs + c1]);
-    uint64_t F0[W];
-    int w0 = 0;
+        const int total = buf.pack(lane, na, a0);
+        if (lane == 0) buf.st[0].arcs += (unsigned)total;
+        // writes the sums of chunk j of the group
+        auto flush = [&](int j) {
+            const int nj = buf.nch[j];
+            const uint32_t *nw = reinterpret_cast<const uint32_t *>(buf.n[j]);
+            T *row = sigma + (size_t)buf.v[j] * S;
 #pragma unroll
-    for (int w = 0; w < W; ++w) F0[w] = 0ull;
-    if (h0) {
-        const uint64_t *vrow = p.vs + (size_t)d0.v * stride;
+            for (int q = 0; q < PL; ++q) {
+                T x = acc[q];
+                over |= SigOver<T>::test(x);
+                if (nj == 1) {
+                    if (nw[q] & lbit) row[32 * q] = x;
+                } else if (x != T(0)) {
+                    x += atomicAdd(row + 32 * q, x);
+                    over |= SigOver<T>::test(x);
+                }
+                flag_two53(p, x, lane + 32 * q);
+                acc[q] = T(0);
+            }
+        };
+        int jc = 0;  // chunk whose sums are in acc
+        int un, jn;
+        jn = buf.find(lane);
+        un = lane < total ? __ldcs(p.rcol + buf.aoff[jn] + lane) : -1;
+        for (int base = 0; base < total; base += 32) {
+            const int u = un, j = jn;
+            uint64_t t[W];
+            if (u >= 0) load_mask<W>(p.vs + (size_t)u * p.vs_stride + prv * W, t);
+            {
+                const int idx = base + 32 + lane;
+                jn = buf.find(idx);
+                un = idx < total ? __ldcs(p.rcol + buf.aoff[jn] + idx) : -1;
+            }
+            bool any = false;
+            if (u >= 0) {
 #pragma unroll
-        for (int w = 0; w < W; ++w) F0[w] = vrow[cur * W + w];
-        w0 = lane < d0.na ? p.col[d0.a0 + lane] : 0;
-    }
-    while (h0) {
-        // chunk i + 2: descriptor; chunk i + 1: frontier mask and first heads
-        Chunk d2{};
-        long long c2 = 0;
-        const bool h2 = h1 && grab.next(c2, lane);
-        if (h2) d2 = load_chunk(&p.chunks[cs + c2]);
-        uint64_t F1[W];
-        int w1 = 0;
+                for (int w = 0; w < W; ++w) {
+                    t[w] &= buf.n[j][w];
+                    any |= t[w] != 0ull;
+                    tight += (unsigned)__popcll(t[w]);
+                    buf.t[lane][w] = t[w];
+                }
+            }
+            unsigned bal = __ballot_sync(kFull, any);
+            __syncwarp();
+            while (bal) {
+                int jj[U];
+                T x[U][PL];
 #pragma unroll
-        for (int w = 0; w < W; ++w) F1[w] = 0ull;
-        if (h1) {
-            const uint64_t *vrow = p.vs + (size_t)d1.v * stride;
+                for (int k = 0; k < U; ++k) {
+                    jj[k] = -1;
+                    if (k == 0 || bal) {
+                        const int i = __ffs(bal) - 1;
+                        bal &= bal - 1;
+                        jj[k] = __shfl_sync(kFull, j, i);
+                        const T *row = sigma + (size_t)__shfl_sync(kFull, u, i) * S;
+                        const uint32_t *tw = reinterpret_cast<const uint32_t *>(buf.t[i]);
 #pragma unroll
-            for (int w = 0; w < W; ++w) F1[w] = vrow[cur * W + w];
-            w1 = lane < d1.na ? p.col[d1.a0 + lane] : 0;
+                        for (int q = 0; q < PL; ++q) x[k][q] = (tw[q] & lbit) ? row[32 * q] : T(0);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    if (k > 0 && jj[k] < 0) break;
+                    if (jj[k] != jc) {
+                        flush(jc);
+                        jc = jj[k];
+                    }
+#pragma unroll
+                    for (int q = 0; q < PL; ++q) acc[q] += x[k][q];
+                }
+            }
+            // at most 32 terms of below 2^26 each since the last test
+#pragma unroll
+            for (int q = 0; q < PL; ++q) over |= SigOver<T>::test(acc[q]);
+            __syncwarp();
         }
-        expand_chunk<W, MODE>(p, L, d0, F0, w0, es1, cs1, ics1, st, s_need);
-        h0 = h1;
-        d0 = d1;
-#pragma unroll
-        for (int w = 0; w < W; ++w) F0[w] = F1[w];
-        w0 = w1;
-        h1 = h2;
-        d1 = d2;
+        flush(jc);
+        __syncwarp();
+    }
+    buf.st[lane].tight += tight;
+    if (over) set_err(p.ctr, kDevWide);
+}
+
+// Bookkeeping of the level-L entries after a bottom-up step (which counts
+// paths itself), one thread each.
+template <int W>
+__device__ void enter_level(const TravParams &p, int L, long long es, long long ecnt, long long gthr,
+                            long long nthr) {
+    Stats &st = warp_buf<W>().st[threadIdx.x & 31];
+    const int own = 1 + (L & 1);
+    for (long long e = es + gthr; e < es + ecnt; e += nthr) {
+        const int v = p.hv[e];
+        const uint64_t *row = p.vs + (size_t)v * p.vs_stride;
+        uint64_t F[W], vis[W];
+        load_mask<W>(row + own * W, F);
+        load_mask<W>(row, vis);
+        enter_entry<W>(p, L, e, v, F, vis, (int)(p.off[v + 1] - p.off[v]), st);
     }
 }
 
 // Bottom-up step of level L (the forward pass of Section 2 read from the
 // other end): sigma_s(v) is the sum of sigma_s(u) over the in-neighbours u
 // of v at level L for s, so every vertex v that some source of the tile has
-// not reached yet (U = valid & ~(visited(v) | current(v))) scans its in-arcs
+// not reached yet (U = valid & ~visited(v)) scans its in-arcs
 // in R(G), and for each in-neighbour u the sources of current(u) & U reach v
 // at level L + 1, each adding sigma_s(u). The sums stay in registers: a
 // vertex whose in-arcs fit one chunk writes its sigma row and its next-level
 // mask once, with no atomic per arc (longer rows are cut into chunks that
-// meet in fp64 atomic adds, exact for integers below 2^53). Lane l holds
-// sources l + 32 i, as in the push. The level-L entries themselves get the
-// bookkeeping the push does for the first chunk of an entry: masks into the
-// history, visited |= F, work counters, query levels and the 2^53 check.
-// Appends are gathered in a per-warp buffer (lane i holds the i-th) and go
-// out 32 at a time through warp_append.
-template <int W, int MODE>
-__device__ __noinline__ void pull_level(const TravParams &p, int L, long long es, long long es1, long long cs1, long long ics1,
-                           Stats &st, const uint64_t *s_need, const uint64_t *s_valid, long long gwarp,
-                           long long nwarps) {
+// meet in atomic adds). Lane l holds sources l + 32 i. The new entries get
+// their bookkeeping from enter_level after the grid barrier that follows.
+template <int W, int MODE, typename T>
+__device__ __noinline__ void pull_level(int L, const uint64_t *s_valid, long long nwarps) {
+    const TravParams &p = shared_params();
+    Stats st;
+    WarpBuf<W> &buf = warp_buf<W>();
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
     const int lane = threadIdx.x & 31;
@@ -442,48 +723,10 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
     const int nxt = 1 + ((L + 1) & 1);
     const int stride = p.vs_stride;
     const int CH = p.chunk_arcs;
-    // (1) the level-L entries, one warp each
-    for (long long e = es + gwarp; e < es1; e += nwarps) {
-        const int v = p.hv[e];
-        const uint64_t *vrow = p.vs + (size_t)v * stride;
-        uint64_t F[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) F[w] = vrow[cur * W + w];
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-            if (lane == w) {
-                p.hm[(size_t)e * W + w] = F[w];
-                atomicOr((unsigned long long *)&p.vs[(size_t)v * stride + w], (unsigned long long)F[w]);
-            }
-        if (lane == 0) {
-            int pc = 0;
-#pragma unroll
-            for (int w = 0; w < W; ++w) pc += __popcll(F[w]);
-            st.edges += (unsigned)pc * (unsigned)(p.off[v + 1] - p.off[v]);
-            st.reached += (unsigned)pc;
-        }
-        const uint64_t qm = p.qmask[v];
-        const double *srow = p.sigma + (size_t)v * S;
-#pragma unroll
-        for (int ii = 0; ii < PL; ++ii) {
-            const int s = lane + 32 * ii;
-            if (mask_bit<W>(F, s)) {
-                if (qm) {
-                    uint64_t x = qm & s_need[s];
-                    while (x) {
-                        const int q = __ffsll((long long)x) - 1;
-                        x &= x - 1;
-                        p.qlevel[s * 64 + q] = L;
-                    }
-                }
-                if (srow[s] >= 9007199254740992.0)
-                    atomicOr((unsigned long long *)&p.srcflag[s >> 6], 1ull << (s & 63));
-            }
-        }
-    }
-    // (2) every vertex's in-arc chunks, handed out dynamically
-    int bv = 0, bnch = 0, binch = 0, bcnt = 0;
-    long long brb = 0, bre = 0, birb = 0, bire = 0;
+    T *sigma = reinterpret_cast<T *>(p.sigma);
+    unsigned over = 0;
+    // every vertex's in-arc chunks, handed out dynamically
+    int qn = 0;  // claimed vertices in the queue
     ChunkGrabber grab(&p.lev_grab[L], p.npchunks, nwarps);
     long long c;
     while (grab.next(c, lane)) {
@@ -494,7 +737,7 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
         bool anyu = false;
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            U[w] = s_valid[w] & ~(vrow[w] | vrow[cur * W + w]);
+            U[w] = s_valid[w] & ~vrow[w];
             anyu |= U[w] != 0ull;
         }
         if (!anyu) continue;  // every source of the tile has reached v
@@ -502,9 +745,9 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
         const long long a0 = rb + (long long)pc.y * CH;
         const int na = (int)min((long long)CH, re - a0);
         const int nch = (int)((re - rb + CH - 1) / CH);
-        double acc[PL];
+        T acc[PL];
 #pragma unroll
-        for (int ii = 0; ii < PL; ++ii) acc[ii] = 0.0;
+        for (int ii = 0; ii < PL; ++ii) acc[ii] = T(0);
         unsigned lm = 0;  // bit ii: source lane + 32 ii reaches v here
         int unext = lane < na ? p.rcol[a0 + lane] : 0;
         for (int base = 0; base < na; base += 32) {
@@ -543,15 +786,16 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
                     n0[w] = __shfl_sync(kFull, t[w], i0);
                     n1[w] = i1 < 0 ? 0ull : __shfl_sync(kFull, t[w], j1);
                 }
-                const double *r0 = p.sigma + (size_t)u0 * S;
-                const double *r1 = p.sigma + (size_t)u1 * S;
+                const T *r0 = sigma + (size_t)u0 * S;
+                const T *r1 = sigma + (size_t)u1 * S;
 #pragma unroll
                 for (int ii = 0; ii < PL; ++ii) {
                     const int s = lane + 32 * ii;
                     const bool b0 = mask_bit<W>(n0, s), b1 = mask_bit<W>(n1, s);
-                    const double x0 = b0 ? r0[s] : 0.0;
-                    const double x1 = b1 ? r1[s] : 0.0;
+                    const T x0 = b0 ? r0[s] : T(0);
+                    const T x1 = b1 ? r1[s] : T(0);
                     acc[ii] += x0 + x1;
+                    over |= SigOver<T>::test(acc[ii]);
                     if (b0 | b1) lm |= 1u << ii;
                 }
             }
@@ -572,40 +816,28 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
         for (int w = 0; w < W; ++w)
             if (lane == w && nm[w])
                 atomicOr((unsigned long long *)&p.vs[(size_t)v * stride + nxt * W + w], (unsigned long long)nm[w]);
-        double *srow = p.sigma + (size_t)v * S;
+        T *srow = sigma + (size_t)v * S;
 #pragma unroll
         for (int ii = 0; ii < PL; ++ii)
             if ((lm >> ii) & 1u) {
+                T x = acc[ii];
                 if (nch == 1)
-                    srow[lane + 32 * ii] = acc[ii];
+                    srow[lane + 32 * ii] = x;
                 else
-                    atomicAdd(&srow[lane + 32 * ii], acc[ii]);
+                    x += atomicAdd(&srow[lane + 32 * ii], x);
+                over |= SigOver<T>::test(x);
+                flag_two53(p, x, lane + 32 * ii);
             }
         int old = 0;
         if (lane == 0) old = atomicMax(&p.tag[v], L + 1);
         old = __shfl_sync(kFull, old, 0);
-        if (old < L + 1) {
-            const long long wrb = p.off[v], wre = p.off[v + 1];
-            if (lane == 0 && old < 0) {
-                st.vb += 1;
-                st.eb += (unsigned)(wre - wrb);
-            }
-            if (lane == bcnt) {
-                bv = v;
-                brb = wrb;
-                bre = wre;
-                bnch = (int)max(1ll, (wre - wrb + CH - 1) / CH);
-                birb = rb;
-                bire = re;
-                binch = MODE == kModeSpd ? nch : 0;
-            }
-            if (++bcnt == 32) {
-                warp_append<W, MODE>(p, L, true, bv, bnch, brb, bre, binch, birb, bire, es1, cs1, ics1, lane);
-                bcnt = 0;
-            }
-        }
+        claim<W>(buf, qn, lane == 0 && old < L + 1, (unsigned)v | (old < 0 ? kFirstSeen : 0u), lane);
+        drain<W, MODE>(L, qn, false);
     }
-    warp_append<W, MODE>(p, L, lane < bcnt, bv, bnch, brb, bre, binch, birb, bire, es1, cs1, ics1, lane);
+    drain<W, MODE>(L, qn, true);
+    buf.st[lane].tight += st.tight;
+    buf.st[lane].arcs += st.arcs;
+    if (over) set_err(p.ctr, kDevWide);
 }
 
 // Eq. 4, push form, from level L into level L - 1: each entry w of level L
@@ -616,15 +848,16 @@ __device__ __noinline__ void pull_level(const TravParams &p, int L, long long es
 // atomic adds. c is formed on the fly from the sigma and acc slabs, which this
 // step only reads for level-L pairs. The in-arc chunks of level L were cut in
 // the forward pass. Lane l holds sources l + 32 i; two tight tails per step.
-template <int W>
+template <int W, typename T>
 __device__ void push_level(const TravParams &p, int L, long long ics, long long ccnt, const uint64_t *s_act,
-                           long long nwarps, Stats &st) {
+                           long long nwarps) {
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
     const int lane = threadIdx.x & 31;
     const int par = 1 + ((L - 1) & 1);  // parity slot holding the level-(L-1) masks
     const int stride = p.vs_stride;
     ChunkGrabber grab(&p.lev_grab[p.maxlev + 2 + L], ccnt, nwarps);
+    unsigned arcs = 0;
     long long c;
     while (grab.next(c, lane)) {
         const Chunk ch = load_chunk(&p.ichunks[ics + c]);
@@ -635,10 +868,11 @@ __device__ void push_level(const TravParams &p, int L, long long ics, long long 
         uint64_t F[W];
 #pragma unroll
         for (int k = 0; k < W; ++k) F[k] = p.hm[(size_t)ch.e * W + k] & s_act[k];
+        const T *sigma = reinterpret_cast<const T *>(p.sigma);
         double sw[PL], aw[PL], cw[PL];
 #pragma unroll
         for (int ii = 0; ii < PL; ++ii) {
-            sw[ii] = p.sigma[(size_t)w * S + lane + 32 * ii];
+            sw[ii] = (double)sigma[(size_t)w * S + lane + 32 * ii];
             aw[ii] = p.acc[(size_t)w * S + lane + 32 * ii];
         }
 #pragma unroll
@@ -657,7 +891,7 @@ __device__ void push_level(const TravParams &p, int L, long long ics, long long 
                     tm[k] = F[k] & row[par * W + k];
                     any |= tm[k] != 0ull;
                 }
-                st.arcs += 1;
+                arcs += 1;
             } else {
 #pragma unroll
                 for (int k = 0; k < W; ++k) tm[k] = 0ull;
@@ -688,6 +922,7 @@ __device__ void push_level(const TravParams &p, int L, long long ics, long long 
             }
         }
     }
+    warp_buf<W>().st[lane].arcs += arcs;
 }
 
 // The rest of a backward step at level L, one thread per entry: delta_s(r_q)
@@ -695,7 +930,7 @@ __device__ void push_level(const TravParams &p, int L, long long ics, long long 
 // complete), and, when the pass goes on, the parity slot shared by levels L
 // and L - 2: the level-L bits leave it and the level-(L - 2) bits enter it
 // (the push from L - 1 reads them in the next step).
-template <int W>
+template <int W, typename T>
 __device__ void level_outputs(const TravParams &p, int L, bool swap, bool set_next, const uint64_t *s_act,
                               const uint64_t *s_need, long long gthr, long long nthr) {
     constexpr int S = 64 * W;
@@ -722,7 +957,7 @@ __device__ void level_outputs(const TravParams &p, int L, bool swap, bool set_ne
                 b &= b - 1;
                 uint64_t x = qm & s_need[s];
                 if (!x) continue;
-                const double d = p.sigma[(size_t)v * S + s] * p.acc[(size_t)v * S + s];
+                const double d = (double)reinterpret_cast<const T *>(p.sigma)[(size_t)v * S + s] * p.acc[(size_t)v * S + s];
                 while (x) {
                     const int q = __ffsll((long long)x) - 1;
                     x &= x - 1;
@@ -754,7 +989,7 @@ __device__ void level_outputs(const TravParams &p, int L, bool swap, bool set_ne
 // a time, each lane adding the terms of its sources l + 32 i in registers.
 // Each warp's sums, times sigma_sr, go to vsum with one fp64 atomic add per
 // source.
-template <int W>
+template <int W, typename T>
 __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_need, long long gwarp,
                             long long nwarps) {
     constexpr int S = 64 * W;
@@ -815,17 +1050,17 @@ __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_nee
                         f0[w] = p.hm[(b + i0) * W + w];
                         f1[w] = p.hm[(b + j1) * W + w];
                     }
-                    const double *q0 = p.sigma + (size_t)t0 * S;
-                    const double *q1 = p.sigma + (size_t)t1 * S;
+                    const T *q0 = reinterpret_cast<const T *>(p.sigma) + (size_t)t0 * S;
+                    const T *q1 = reinterpret_cast<const T *>(p.sigma) + (size_t)t1 * S;
 #pragma unroll
                     for (int ii = 0; ii < PL; ++ii) {
                         const int s = lane + 32 * ii;
                         if (ks[ii] == k0 && mask_bit<W>(f0, s)) {
-                            a[ii] += r0 / q0[s];
+                            a[ii] += r0 / (double)q0[s];
                             ++pairs;
                         }
                         if (ks[ii] == k1 && mask_bit<W>(f1, s)) {
-                            a[ii] += r1 / q1[s];
+                            a[ii] += r1 / (double)q1[s];
                             ++pairs;
                         }
                     }
@@ -833,14 +1068,23 @@ __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_nee
             }
         }
     }
-    const double *sr = p.sigma + (size_t)p.vroot * S;
+    const T *sr = reinterpret_cast<const T *>(p.sigma) + (size_t)p.vroot * S;
 #pragma unroll
     for (int ii = 0; ii < PL; ++ii)
-        if (a[ii] != 0.0) atomicAdd(&p.vsum[lane + 32 * ii], sr[lane + 32 * ii] * a[ii]);
+        if (a[ii] != 0.0) atomicAdd(&p.vsum[lane + 32 * ii], (double)sr[lane + 32 * ii] * a[ii]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(kFull, pairs, o);
     if (lane == 0 && pairs) atomicAdd(&p.ctr->vpairs, (unsigned long long)pairs);
 }
+
+// Shared sums of vertex_scan_multi (in the space the warps' buffers take
+// during the forward pass).
+template <int W>
+struct ScanBuf {
+    static constexpr int G = W >= 8 ? 4 : 8;  // columns per pass
+    double acc[64 * W * G];                   // [s][column]
+    int32_t ql[64 * W * G];                   // d(s, r_c) for sources that need column c, else -1
+};
 
 // Dependencies on several query vertices at once by the vertex scan: the
 // form of vertex_scan for a group whose queries sit at up to 64 distinct
@@ -855,14 +1099,16 @@ __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_nee
 // shared sums [s][c]; at the end of the 8 columns the block multiplies them by
 // sigma_s(r_c) and adds them into msum [s * 64 + c] with one fp64 atomic each.
 // No level order and no grid barrier inside.
-template <int W>
-__device__ __noinline__ void vertex_scan_multi(const TravParams &p, int Lmax, const uint64_t *s_need, long long gwarp,
-                                               long long nwarps) {
+template <int W, typename T>
+__device__ __noinline__ void vertex_scan_multi(int Lmax, long long gwarp, long long nwarps) {
+    const TravParams &p = shared_params();
+    const uint64_t *s_need = tile_need();
+    ScanBuf<W> &sb = *reinterpret_cast<ScanBuf<W> *>(s_dyn + kParamBytes + 512 * W);
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
-    constexpr int G = W >= 8 ? 4 : 8;  // columns per pass (the shared sums of 512 sources x 8 columns would pass 48 KB)
-    __shared__ double s_acc[S * G];
-    __shared__ int32_t s_ql[S * G];  // d(s, r_c) for sources that need column c, else -1
+    constexpr int G = ScanBuf<W>::G;
+    double *const s_acc = sb.acc;
+    int32_t *const s_ql = sb.ql;
     __shared__ int32_t s_kmin[G], s_kmax[G];
     __shared__ unsigned long long s_kset[G];
     const int lane = threadIdx.x & 31;
@@ -945,7 +1191,7 @@ __device__ __noinline__ void vertex_scan_multi(const TravParams &p, int Lmax, co
                     uint64_t F[W];
 #pragma unroll
                     for (int w = 0; w < W; ++w) F[w] = p.hm[(b + i) * W + w];
-                    const double *qs = p.sigma + (size_t)ti * S;
+                    const T *qs = reinterpret_cast<const T *>(p.sigma) + (size_t)ti * S;
                     while (kqi) {
                         const int j = __ffs(kqi) - 1;
                         kqi &= kqi - 1;
@@ -959,7 +1205,7 @@ __device__ __noinline__ void vertex_scan_multi(const TravParams &p, int Lmax, co
                         for (int ii = 0; ii < PL; ++ii) {
                             const int s = lane + 32 * ii;
                             if (mask_bit<W>(F, s) && s_ql[s * G + j] == k) {
-                                atomicAdd(&s_acc[s * G + j], rs / qs[s]);
+                                atomicAdd(&s_acc[s * G + j], rs / (double)qs[s]);
                                 ++pairs;
                             }
                         }
@@ -973,7 +1219,7 @@ __device__ __noinline__ void vertex_scan_multi(const TravParams &p, int Lmax, co
             const double a = s_acc[i];
             if (a != 0.0) {
                 const int sl = i / G, j = i % G;
-                atomicAdd(&p.msum[sl * 64 + cg + j], a * p.sigma[(size_t)p.croot[cg + j] * S + sl]);
+                atomicAdd(&p.msum[sl * 64 + cg + j], a * (double)reinterpret_cast<const T *>(p.sigma)[(size_t)p.croot[cg + j] * S + sl]);
             }
         }
     }
@@ -982,31 +1228,79 @@ __device__ __noinline__ void vertex_scan_multi(const TravParams &p, int Lmax, co
     if (lane == 0 && pairs) atomicAdd(&p.ctr->vpairs, (unsigned long long)pairs);
 }
 
-template <int W, int MODE, int MINB>
-__global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
+// The launch's parameters into shared memory, with the state arrays of the
+// block's team: each team has the state of one tile.
+template <typename T>
+__device__ __forceinline__ void load_params(const TravParams &launch, int team) {
+    for (int i = threadIdx.x; i < (int)(sizeof(TravParams) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(s_dyn)[i] = reinterpret_cast<const uint32_t *>(&launch)[i];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        TravParams &p = *reinterpret_cast<TravParams *>(s_dyn);
+        const size_t t = (size_t)team, n = (size_t)p.n, lev = (size_t)p.maxlev + 2, ws = (size_t)p.ws_slots;
+        p.bar += t;
+        p.vs += t * n * p.vs_stride;
+        p.tag += t * n;
+        p.sigma = reinterpret_cast<double *>(reinterpret_cast<T *>(p.sigma) + t * n * ws);
+        p.acc += t * n * ws;
+        p.hv += t * (size_t)p.hcap;
+        p.hm += t * (size_t)p.hm_words;
+        p.chunks += t * (size_t)p.ccap;
+        p.ichunks += t * (size_t)p.ccap;
+        p.lev_cnt += t * lev;
+        p.lev_ccnt += t * lev;
+        p.lev_grab += t * 6 * lev;
+        p.lev_start += t * lev;
+        p.lev_cstart += t * lev;
+        p.lev_icstart += t * lev;
+        p.qlevel += t * ws * 64;
+        p.dep += t * ws * 64;
+        p.vsum += t * 2 * ws;
+        p.msum += t * 2 * ws * 64;
+        p.srcflag += t * (size_t)max(p.ws_slots / 64, 4);
+    }
+    __syncthreads();
+}
+
+// Barrier of the blocks of a team (a lone block needs no wait on others; it
+// still leaves when another team has flagged an error).
+__device__ __forceinline__ bool team_barrier(const TravParams &p, uint32_t &gen) {
+    return grid_barrier(p.ctr, gen, p.timeout_ns, &p.bar->count, &p.bar->gen, (uint32_t)p.team_blocks);
+}
+
+template <int W, int MODE, int MINB, typename T>
+__global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__ TravParams launch) {
     constexpr int S = 64 * W;
+    constexpr int kGatherU = (W <= 2 || (W == 4 && MINB == 1 && sizeof(T) == 4)) ? 2 : 1;  // rows in flight per warp of the gather
+    constexpr int kPushU = W * MINB > 4 ? 1 : 2;                                            // arcs in flight per lane of the push
     const int lane = threadIdx.x & 31;
+    const int team = blockIdx.x / launch.team_blocks;
+    const int block = blockIdx.x - team * launch.team_blocks;  // within the team
+    const bool leader = block == 0 && threadIdx.x == 0;
+    load_params<T>(launch, team);
+    const TravParams &p = shared_params();
+    T *sigma = reinterpret_cast<T *>(p.sigma);
     const long long wpb = blockDim.x >> 5;
-    const long long gwarp = (long long)blockIdx.x * wpb + (threadIdx.x >> 5);
-    const long long nwarps = (long long)gridDim.x * wpb;
-    const long long gthr = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nthr = (long long)gridDim.x * blockDim.x;
+    const long long gwarp = (long long)block * wpb + (threadIdx.x >> 5);
+    const long long nwarps = (long long)p.team_blocks * wpb;
+    const long long gthr = (long long)block * blockDim.x + threadIdx.x;
+    const long long nthr = (long long)p.team_blocks * blockDim.x;
     uint32_t gen = 0;
-    __shared__ uint64_t s_need[S];
+    uint64_t *const s_need = tile_need();
     __shared__ int32_t s_minql[S];
     __shared__ uint64_t s_active[W];
     __shared__ uint64_t s_active_next[W];
     __shared__ uint64_t s_valid[W];  // the tile's occupied source slots
     __shared__ int32_t s_lstop;
-    Stats st;
-    const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
+    const bool timer = team == 0 && leader;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
     unsigned long long ns_fwd = 0, ns_bwd = 0, ns_other = 0;
 
-    for (long long tile = 0; tile < p.ntiles; ++tile) {
+    // a team's first tile is its own number, the next ones come from a counter
+    for (long long tile = team; tile < p.ntiles; tile = (long long)ld_vol(&p.bar->next)) {
         const int32_t *tsrc = p.srcs + tile * S;
         check_cancel(p);
-        if (blockIdx.x == 0) init_tile<W, MODE>(p, tsrc);
+        if (block == 0) init_tile<W, MODE, T>(p, tsrc);
         for (int s = threadIdx.x; s < S; s += blockDim.x) {
             const int32_t v = tsrc[s];
             s_need[s] = (MODE != kModeReach && v >= 0) ? p.need[v] : 0ull;
@@ -1017,7 +1311,8 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
                 if (tsrc[threadIdx.x * 64 + b] >= 0) m |= 1ull << b;
             s_valid[threadIdx.x] = m;
         }
-        if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+        warp_buf<W>().st[lane] = Stats();
+        if (!team_barrier(p, gen)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
@@ -1029,13 +1324,13 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
         int L = 0;
         long long total = 0;
         for (;;) {
-            // the level's entries and chunks, counted in one word by warp_append
+            // the level's entries and chunks, counted in one word by append_queue
             const unsigned long long pk = ld_vol(&p.lev_grab[4 * ((long long)p.maxlev + 2) + L]);
             const long long ecnt = (long long)(pk & 0xffffffffull);
             const long long ccnt = (long long)(pk >> 32);
             const long long iccnt = (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + L]);
             const long long es1 = es + ecnt, cs1 = cs + ccnt, ics1 = ics + iccnt;
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (leader) {
                 p.lev_cnt[L] = (unsigned long long)ecnt;  // published for the passes after the forward
                 p.lev_ccnt[L] = (unsigned long long)ccnt;
                 p.lev_start[L] = es;
@@ -1059,18 +1354,34 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
             // reach the threshold (the same counter in every block)
             const bool pull = MODE != kModeReach && L >= 1 && p.pull_arcs_min > 0 &&
                               (long long)ld_vol(&p.lev_grab[3 * ((long long)p.maxlev + 2) + L]) >= p.pull_arcs_min;
-            if (pull) {
-                pull_level<W, MODE>(p, L, es, es1, cs1, ics1, st, s_need, s_valid, gwarp, nwarps);
-                if (timer) atomicAdd(&p.ctr->pull_levels, 1ull);
-            } else {
-                forward_level<W, MODE, MINB == 1>(p, L, cs, ccnt, es1, cs1, ics1, st, s_need, gwarp, nwarps);
+            if (lane == 0) {
+                warp_buf<W>().first = cs;
+                warp_buf<W>().ends = LevelEnds{es1, cs1, ics1};
             }
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            __syncwarp();
+            if (pull) {
+                pull_level<W, MODE, T>(L, s_valid, nwarps);
+                if (leader) atomicAdd(&p.ctr->pull_levels, 1ull);
+            } else {
+                push_masks<W, MODE, kPushU>(L, ccnt, gwarp, nwarps);
+            }
+            if (!team_barrier(p, gen)) return;
             total = es1;
-            if ((ld_vol(&p.lev_grab[4 * ((long long)p.maxlev + 2) + L + 1]) & 0xffffffffull) == 0ull) break;
+            const long long enext =
+                (long long)(ld_vol(&p.lev_grab[4 * ((long long)p.maxlev + 2) + L + 1]) & 0xffffffffull);
+            if (enext == 0) break;
             if (L + 2 > p.maxlev) {
                 if (threadIdx.x == 0) set_err(p.ctr, kDevLevelOverflow);
                 return;
+            }
+            if (MODE != kModeReach) {
+                if (pull)
+                    enter_level<W>(p, L + 1, es1, enext, gthr, nthr);
+                else if constexpr (MODE != kModeReach)
+                    gather_level<W, T, kGatherU>(
+                        L + 1, ics1, (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + L + 1]), gwarp,
+                        nwarps);
+                if (!team_barrier(p, gen)) return;
             }
             es_prev = es;
             es = es1;
@@ -1083,8 +1394,11 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
             const unsigned long long t = global_ns();
             ns_fwd += t - t_mark;
             t_mark = t;
-            atomicMax(&p.ctr->levels_max, (unsigned long long)Lmax);
         }
+        if (leader) atomicMax(&p.ctr->levels_max, (unsigned long long)Lmax);
+
+        // the scan over several query vertices takes the warps' buffers
+        if (MODE == kModeScan) flush_stats(p.ctr, warp_buf<W>().st[lane], lane);
 
         // ---------------- backward ----------------
         if (MODE == kModeScan && (p.flags & kFlagRootOut)) {
@@ -1100,21 +1414,21 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
                             const int c = __ffsll((long long)x) - 1;
                             x &= x - 1;
                             p.rlevq[(size_t)v * 64 + c] = Lr;
-                            p.rsigq[(size_t)v * 64 + c] = p.sigma[(size_t)v * S + c];
+                            p.rsigq[(size_t)v * 64 + c] = (double)sigma[(size_t)v * S + c];
                         }
                     } else {
                         p.rlev[v] = Lr;
-                        p.rsig[v] = p.sigma[(size_t)v * S];
+                        p.rsig[v] = (double)sigma[(size_t)v * S];
                     }
                 }
             }
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            if (!team_barrier(p, gen)) return;
         } else if (MODE == kModeScan && !(p.flags & kFlagNoBackward)) {
             if (p.ncols >= 2)
-                vertex_scan_multi<W>(p, Lmax, s_need, gwarp, nwarps);
+                vertex_scan_multi<W, T>(Lmax, gwarp, nwarps);
             else
-                vertex_scan<W>(p, Lmax, s_need, gwarp, nwarps);
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                vertex_scan<W, T>(p, Lmax, s_need, gwarp, nwarps);
+            if (!team_barrier(p, gen)) return;
         }
         if (MODE == kModeSpd && !(p.flags & kFlagNoBackward)) {
             if (threadIdx.x == 0) s_lstop = 0x7fffffff;
@@ -1150,7 +1464,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
                         for (int w = 0; w < W; ++w)
                             atomicOr((unsigned long long *)&row[slot * W + w], (unsigned long long)p.hm[e * W + w]);
                     }
-                    if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                    if (!team_barrier(p, gen)) return;
                 }
                 for (int Lb = Lmax; Lb >= lstop; --Lb) {
                     if (threadIdx.x < W) {
@@ -1165,13 +1479,13 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
                     }
                     __syncthreads();
                     const bool more = Lb > lstop;
-                    level_outputs<W>(p, Lb, more, more && Lb - 2 >= lstop, s_active, s_need, gthr, nthr);
+                    level_outputs<W, T>(p, Lb, more, more && Lb - 2 >= lstop, s_active, s_need, gthr, nthr);
                     if (more) {
                         const long long ics = p.lev_icstart[Lb];
                         const long long ic = (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + Lb]);
-                        push_level<W>(p, Lb, ics, ic, s_active_next, nwarps, st);
+                        push_level<W, T>(p, Lb, ics, ic, s_active_next, nwarps);
                     }
-                    if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                    if (!team_barrier(p, gen)) return;
                 }
             }
         }
@@ -1181,10 +1495,10 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
             t_mark = t;
         }
 
-        if (MODE != kModeReach) flush_stats(p.ctr, st, lane);
+        if (MODE == kModeSpd) flush_stats(p.ctr, warp_buf<W>().st[lane], lane);
 
         // ---------------- tile end ----------------
-        if (MODE == kModeScan && blockIdx.x == 0) {
+        if (MODE == kModeScan && block == 0) {
             // one sum per source (one query vertex) or per (source, column)
             for (int s = threadIdx.x; s < S; s += blockDim.x) {
                 uint64_t x = s_need[s];
@@ -1197,33 +1511,49 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
             }
             __syncthreads();
         }
-        if (MODE != kModeReach && blockIdx.x == 0) tile_query_sums(p, tile, S, tsrc, s_need);
+        if (MODE != kModeReach && block == 0) tile_query_sums(p, tile, S, tsrc, s_need);
         if (MODE == kModeReach) {
             for (long long e = gthr; e < total; e += nthr)
                 atomicOr((unsigned long long *)&p.rvmask[p.hv[e]], (unsigned long long)p.hm[e * W]);
         }
         if (!(p.flags & kFlagNoReset)) {
-            for (long long e = gwarp; e < total; e += nwarps) {
-                const int v = p.hv[e];
-                if (MODE != kModeReach) {
-                    uint64_t F[W];
+            if (MODE != kModeReach) {
+                // sigma rows of more than one in-arc chunk meet in atomic adds
+                // and start from zero; the others are overwritten when reached
+                for (long long b = 32 * gwarp; b < total; b += 32 * nwarps) {
+                    const long long e = b + lane;
+                    const int v = e < total ? p.hv[e] : -1;
+                    unsigned lg = __ballot_sync(kFull, v >= 0 && p.roff[v + 1] - p.roff[v] > p.chunk_arcs);
+                    if (MODE == kModeSpd) lg = __ballot_sync(kFull, v >= 0);
+                    while (lg) {
+                        const int i = __ffs(lg) - 1;
+                        lg &= lg - 1;
+                        const int vi = __shfl_sync(kFull, v, i);
+                        T *row = sigma + (size_t)vi * S;
+                        double *arow = p.acc + (size_t)vi * S;
+                        uint64_t F[W];
 #pragma unroll
-                    for (int w = 0; w < W; ++w) F[w] = p.hm[e * W + w];
-                    double *row = p.sigma + (size_t)v * S;
-                    double *arow = p.acc + (size_t)v * S;
+                        for (int w = 0; w < W; ++w) F[w] = p.hm[(b + i) * W + w];
 #pragma unroll
-                    for (int ii = 0; ii < 2 * W; ++ii) {
-                        const int s = lane + 32 * ii;
-                        if (mask_bit<W>(F, s)) {
-                            row[s] = 0.0;
-                            if (MODE == kModeSpd) arow[s] = 0.0;
+                        for (int ii = 0; ii < 2 * W; ++ii) {
+                            const int s = lane + 32 * ii;
+                            if (mask_bit<W>(F, s)) {
+                                row[s] = T(0);
+                                if (MODE == kModeSpd) arow[s] = 0.0;
+                            }
                         }
                     }
                 }
-                if (lane < p.vs_stride) p.vs[(size_t)v * p.vs_stride + lane] = 0ull;
-                if (lane == 0) p.tag[v] = -1;
             }
-            if (blockIdx.x == 0) {
+            const int half = p.vs_stride / 2;  // 16-byte pieces of a vertex's masks
+            for (long long i = gthr; i < total * half; i += nthr) {
+                const long long e = i / half;
+                const int k = (int)(i - e * half);
+                const int v = p.hv[e];
+                reinterpret_cast<ulonglong2 *>(p.vs + (size_t)v * p.vs_stride)[k] = make_ulonglong2(0ull, 0ull);
+                if (k == 0) p.tag[v] = -1;
+            }
+            if (block == 0) {
                 for (int l = threadIdx.x; l <= Lmax + 1; l += blockDim.x) {
                     p.lev_cnt[l] = 0ull;
                     p.lev_ccnt[l] = 0ull;
@@ -1232,10 +1562,12 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
                     p.lev_grab[2 * (p.maxlev + 2) + l] = 0ull;
                     p.lev_grab[3 * (p.maxlev + 2) + l] = 0ull;
                     p.lev_grab[4 * (p.maxlev + 2) + l] = 0ull;
+                    p.lev_grab[5 * (p.maxlev + 2) + l] = 0ull;
                 }
             }
         }
-        if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+        if (leader) *(volatile unsigned long long *)&p.bar->next = p.nteams + atomicAdd(&p.ctr->tiles_taken, 1ull);
+        if (!team_barrier(p, gen)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
@@ -1250,20 +1582,87 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(TravParams p) {
     }
 }
 
-template <int W, int MODE, int MINB>
+template <int W, int MODE, int MINB, typename T>
 bc_status launch(bc_graph *g, TravParams &p) {
-    auto kern = trav_kernel<W, MODE, MINB>;
+    auto kern = trav_kernel<W, MODE, MINB, T>;
     const int threads = g->block_threads;
     if (threads < 64 * W) return set_error(BC_E_INVALID_ARG, "block_threads must be at least 64 * tile_words");
-    const size_t smem = 0;
+    size_t smem = sizeof(WarpBuf<W>) * (size_t)(threads / 32);
+    if (MODE == kModeScan) smem = std::max(smem, sizeof(ScanBuf<W>));
+    smem += kParamBytes + 512 * W;
     int per_sm = 0;
+    BCD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) return set_error(BC_E_INTERNAL, "traversal kernel cannot be resident");
-    dim3 grid((unsigned)(g->num_sms * per_sm)), block((unsigned)threads);
+    const int blocks = g->num_sms * per_sm;
+    p.nteams = (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min(g->ws.teams, blocks), p.ntiles));
+    p.team_blocks = blocks / p.nteams;
+    dim3 grid((unsigned)(p.nteams * p.team_blocks)), block((unsigned)threads);
+    BCD_CUDA(cudaMemsetAsync(p.bar, 0, sizeof(TeamBar) * (size_t)p.nteams, g->stream));
     void *args[] = {(void *)&p};
     BCD_CUDA(cudaLaunchCooperativeKernel((const void *)kern, grid, block, args, smem, g->stream));
     g->launches += 1;
     g->last_grid = (int)grid.x;
+    return BC_OK;
+}
+
+// Launch with path counts as 32-bit integers, or in fp64 once a launch of
+// this graph met a count of 2^26 (rare: the fp64 kernels come at one
+// occupancy each).
+template <int MODE>
+bc_status launch_counts(bc_graph *g, int W, TravParams &p) {
+    const int b = g->blocks_per_sm;
+    if (g->ws.swide) {
+        switch (W) {
+            case 1: return launch<1, MODE, 2, double>(g, p);
+            case 2: return launch<2, MODE, 2, double>(g, p);
+            case 4: return launch<4, MODE, 1, double>(g, p);
+            case 8: return launch<8, MODE, 1, double>(g, p);
+        }
+    } else {
+        switch (W) {
+            case 1: return launch<1, MODE, 2, uint32_t>(g, p);
+            case 2: return b == 3 ? launch<2, MODE, 3, uint32_t>(g, p) : launch<2, MODE, 2, uint32_t>(g, p);
+            case 4: return b == 2 ? launch<4, MODE, 2, uint32_t>(g, p) : launch<4, MODE, 1, uint32_t>(g, p);
+            case 8: return launch<8, MODE, 1, uint32_t>(g, p);
+        }
+    }
+    return set_error(BC_E_INVALID_ARG, "tile words must be 1, 2, 4 or 8");
+}
+
+// The state slabs of an unweighted launch. The sigma slab starts with the rows
+// of several in-arc chunks zero: the row width, the count type and chunk_arcs
+// decide which rows these are and where they lie, so a change of any of them
+// clears the slab (and fp64 counts need a larger one). The accumulators of
+// Eq. 4 start zero.
+bc_status prepare_slabs(bc_graph *g, int W, bool eq4) {
+    bcd_workspace &ws = g->ws;
+    const size_t pairs = (size_t)ws.teams * (size_t)ws.n * 64 * (size_t)ws.W;
+    const size_t bytes = ws.swide ? sizeof(double) : sizeof(uint32_t);
+    if (ws.sigma_bytes < bytes) {
+        dev_free(ws.sigma);
+        ws.sigma_key = -1;
+        ws.sigma_zero = false;
+        const bc_status st = dev_alloc(&ws.sigma, pairs);
+        if (st != BC_OK) {
+            free_workspace(g);
+            return st;
+        }
+        ws.sigma_bytes = bytes;
+    }
+    const int64_t key = ((int64_t)g->chunk_arcs << 8) | (int64_t)(W << 1) | (ws.swide ? 1 : 0);
+    if (ws.sigma_key != key && !ws.sigma_zero)
+        BCD_CUDA(cudaMemsetAsync(ws.sigma, 0, ws.sigma_bytes * pairs, g->stream));
+    ws.sigma_key = key;
+    ws.sigma_zero = false;
+    if (eq4 && !ws.acc) {
+        const bc_status st = dev_alloc(&ws.acc, pairs);
+        if (st != BC_OK) {
+            free_workspace(g);
+            return st;
+        }
+        BCD_CUDA(cudaMemsetAsync(ws.acc, 0, sizeof(double) * pairs, g->stream));
+    }
     return BC_OK;
 }
 
@@ -1272,14 +1671,16 @@ bc_status launch(bc_graph *g, TravParams &p) {
 bc_status reset_dense_state(bc_graph *g) {
     bcd_workspace &ws = g->ws;
     if (!ws.vs) return BC_OK;  // no workspace (never built, or freed after a failure)
-    BCD_CUDA(cudaMemsetAsync(ws.vs, 0, sizeof(uint64_t) * (size_t)ws.n * ws.vs_stride, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.tag, 0xff, sizeof(int32_t) * (size_t)ws.n, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.sigma, 0, sizeof(double) * (size_t)ws.n * 64 * ws.W, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.lev_cnt, 0, sizeof(unsigned long long) * (size_t)(ws.maxlev + 2), g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.lev_ccnt, 0, sizeof(unsigned long long) * (size_t)(ws.maxlev + 2), g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.lev_grab, 0, sizeof(unsigned long long) * 6 * (size_t)(ws.maxlev + 2), g->stream));
+    const size_t t = (size_t)ws.teams, n = (size_t)ws.n, lev = (size_t)(ws.maxlev + 2);
+    BCD_CUDA(cudaMemsetAsync(ws.vs, 0, sizeof(uint64_t) * t * n * ws.vs_stride, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.tag, 0xff, sizeof(int32_t) * t * n, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.sigma, 0, ws.sigma_bytes * t * n * 64 * ws.W, g->stream));
+    ws.sigma_zero = true;
+    BCD_CUDA(cudaMemsetAsync(ws.lev_cnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.lev_ccnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.lev_grab, 0, sizeof(unsigned long long) * t * 6 * lev, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.pdone, 0, sizeof(int32_t) * (size_t)(g->weighted ? ws.pcap : 1), g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.acc, 0, sizeof(double) * (g->weighted ? (size_t)1 : (size_t)ws.n * 64 * ws.W), g->stream));
+    if (ws.acc) BCD_CUDA(cudaMemsetAsync(ws.acc, 0, sizeof(double) * t * n * 64 * ws.W, g->stream));
     if (ws.dist) {
         BCD_CUDA(cudaMemsetAsync(ws.dist, 0xff, sizeof(uint64_t) * (size_t)ws.n * 64 * ws.W, g->stream));
         BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 2 * (size_t)ws.ring, g->stream));
@@ -1290,6 +1691,7 @@ bc_status reset_dense_state(bc_graph *g) {
 bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsigned long long *edges_out) {
     for (int attempt = 0; attempt < 6; ++attempt) {
         bcd_workspace &ws = g->ws;
+        if (!g->weighted && p.mode != kModeReach) BCD_TRY(prepare_slabs(g, W, p.mode == kModeSpd));
         p.vs = ws.vs;
         p.vs_stride = ws.vs_stride;
         p.tag = ws.tag;
@@ -1300,6 +1702,11 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         p.hv = ws.hv;
         p.hm = ws.hm;
         p.hcap = p.mode == kModeReach ? ws.hmcap : ws.hcap;
+        p.hm_words = ws.hcap * ws.W;
+        p.ws_slots = 64 * ws.W;
+        p.bar = ws.bar;
+        p.nteams = 1;
+        p.team_blocks = 1;
         p.chunks = ws.chunks;
         p.ichunks = ws.ichunks;
         p.ccap = ws.ccap;
@@ -1332,7 +1739,7 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         if (timed) cudaEventRecord(ev0, g->stream);
         if (p.mode == kModeReach) {
             if (W != 1) return set_error(BC_E_INTERNAL, "reach traversal runs with one mask word");
-            st = launch<1, kModeReach, 2>(g, p);
+            st = launch<1, kModeReach, 2, uint32_t>(g, p);
         } else if (g->weighted) {
             p.wt = g->d_w;
             p.roff = g->d_roff;
@@ -1350,27 +1757,8 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
             p.wshort = g->wshort;
             p.lev_dist = ws.lev_dist;
             st = launch_weighted(g, p);
-        } else if (p.mode == kModeScan) {
-            if (W == 1)
-                st = launch<1, kModeScan, 2>(g, p);
-            else if (W == 2)
-                st = g->blocks_per_sm == 3 ? launch<2, kModeScan, 3>(g, p) : launch<2, kModeScan, 2>(g, p);
-            else if (W == 4)
-                st = g->blocks_per_sm == 2 ? launch<4, kModeScan, 2>(g, p) : launch<4, kModeScan, 1>(g, p);
-            else if (W == 8)
-                st = launch<8, kModeScan, 1>(g, p);
-            else
-                return set_error(BC_E_INVALID_ARG, "tile words must be 1, 2, 4 or 8");
-        } else if (W == 1) {
-            st = launch<1, kModeSpd, 2>(g, p);
-        } else if (W == 2) {
-            st = g->blocks_per_sm == 3 ? launch<2, kModeSpd, 3>(g, p) : launch<2, kModeSpd, 2>(g, p);
-        } else if (W == 4) {
-            st = g->blocks_per_sm == 2 ? launch<4, kModeSpd, 2>(g, p) : launch<4, kModeSpd, 1>(g, p);
-        } else if (W == 8) {
-            st = launch<8, kModeSpd, 1>(g, p);
         } else {
-            return set_error(BC_E_INVALID_ARG, "tile words must be 1, 2, 4 or 8");
+            st = p.mode == kModeScan ? launch_counts<kModeScan>(g, W, p) : launch_counts<kModeSpd>(g, W, p);
         }
         if (timed) cudaEventRecord(ev1, g->stream);
         if (st != BC_OK) {
@@ -1405,6 +1793,13 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         if (c.err == kDevCancelled) {
             reset_dense_state(g);
             return set_error(BC_E_CANCELLED, "traversal: cancelled by bc_cancel");
+        }
+        if (c.err == kDevWide) {
+            // a path count of 2^26: fp64 counts from now on
+            ws.swide = true;
+            BCD_TRY(reset_dense_state(g));
+            if (p.qflags) BCD_CUDA(cudaMemsetAsync(p.qflags, 0, sizeof(uint32_t) * 64, g->stream));
+            continue;
         }
         if (c.err == kDevBucketOverflow) {
             // more pending pairs at one distance than a ring slot holds: grow and rerun
