@@ -410,12 +410,13 @@ void bc_server_destroy(bc_server *srv);
  *                  (the 64 * weighted_words sources of a tile settle their
  *                  (vertex, source) pairs together, one grid-wide barrier
  *                  per distance value); 2 (default) the source kernel: each
- *                  block (1024 threads, one per SM; block_threads does not
+ *                  block (256 to 1024 threads, four to one per SM, by the
+ *                  number of vertices; block_threads does not
  *                  apply) takes one source at a time and settles its
  *                  distances with block barriers only, so blocks never wait
  *                  on one another (per block: 20 bytes per vertex plus the
  *                  bucket ring; as many blocks as fit in half of the free
- *                  device memory, up to one per SM). Both give
+ *                  device memory, up to the residency above). Both give
  *                  the same distances and sigma; dependencies agree up to
  *                  fp64 summation order. The traversal rooted at the query
  *                  vertices of the vertex scan, and bc_spd_probe, always

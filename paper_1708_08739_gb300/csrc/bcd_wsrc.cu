@@ -29,19 +29,24 @@
 // pair holds its distance with the sum over exactly its tight in-arcs (sigma
 // values are integers: exact in any order below 2^53). Every arc is read
 // once in the forward pass, along its tail's out-row; no in-arc pass.
+// Where it fits, shared memory holds one bit per vertex: settled for the
+// current source. An arc to a settled vertex can change nothing, and most arcs
+// are such (they lead to hubs, which settle early), so their heads' distances,
+// random 32-byte sectors each, are not read.
 // A vertex queued in the slot of d whose distance has since dropped is stale
 // and skipped; a vertex is queued only when its distance strictly drops, so
 // it settles once.
 //
-// A level's queued vertices are spread over the block's lanes, 1 to 32 lanes
-// per vertex (as many as the level's size leaves room for); each lane walks
-// every LPP-th arc. Vertices with more than weighted_short_row out-arcs are
-// cut into chunk_arcs chunks that warps take after a block barrier (lanes
-// over arcs). The source is flagged when a sigma reaches 2^53. The Eq. 4
-// pass walks the levels from the deepest to the shallowest level holding a
-// query vertex the source serves, summing c over tight out-arcs (short rows
-// by LPP lanes and a fixed shuffle tree, long rows by chunks added in chunk
-// order), so delta is the same from run to run.
+// A level's queued vertices go to the warps in groups of up to 32, and a warp
+// packs the out-arcs of its group onto its lanes (four arcs per lane in
+// flight), so a level costs its arcs and not its longest row. Rows of more than
+// kPackRows * weighted_short_row arcs are cut into chunk_arcs chunks that all
+// warps take after a block barrier. The source is flagged when a sigma reaches
+// 2^53. The Eq. 4 pass walks the levels from the deepest to the shallowest
+// level holding a query vertex the source serves, summing c over tight
+// out-arcs: it reads a vertex's arc bits 32 at a time and visits only the arcs
+// whose bit is set (a row by 1 to 32 lanes and a fixed shuffle tree, longer
+// rows by chunks added in chunk order), so delta is the same from run to run.
 //
 // Each source's dependencies delta_s.(r_q) go to sdep[i * 64 + q] (i its
 // position in the launch's source list, q the queries that need it); a
@@ -63,10 +68,16 @@ namespace {
 using namespace dev;
 
 constexpr int kLanesBatch = 4;  // arcs a lane loads together
-// One block of 1024 threads per SM: fewer sources in flight, each with more
-// lanes, measured faster than two blocks of 512 or four of 256 (a smaller
-// footprint of per-source state, and shorter per-level chains)
+constexpr int kPullBatch = 2;   // ... in the Eq. 4 pass, of those whose bit is set
+// Rows of up to this many times weighted_short_row arcs are packed with their
+// group's (forward) or walked by their lanes (backward); longer ones are cut.
+constexpr int kPackRows = 4;
+// Threads of the largest block (one per SM at 64 registers); see src_threads.
 constexpr int kSrcThreads = 1024;
+// Dynamic shared memory of a block (227 KB less the static arrays): the warps'
+// staging, the ring's counters and, up to about 1.6 million vertices, the
+// settled bits.
+constexpr size_t kSrcDynSmem = 224 * 1024;
 constexpr double kSrcTwo53 = 9007199254740992.0;
 
 // (distance, sigma) of one vertex for the block's current source
@@ -157,7 +168,10 @@ struct WidePairs {
         x.s = 0.0;
         ds[v] = x;
     }
-    __device__ __forceinline__ int offer(int v, unsigned long long nd, double sg) const {
+    using Seen = unsigned long long;  // what a first look at a head loads: its distance
+    __device__ __forceinline__ Seen look(int v) const { return ds[v].d; }
+    static __device__ __forceinline__ unsigned long long dist_of(Seen x) { return x; }
+    __device__ __forceinline__ int offer(int v, unsigned long long nd, double sg, Seen) const {
         DistSig *q = ds + v;
         DistSig cur = *q;
         for (int it = 0; it < kCasTries; ++it) {
@@ -191,10 +205,12 @@ struct NarrowPairs {
     }
     __device__ __forceinline__ void seed(int v) const { w[v] = 1ull << 24; }
     __device__ __forceinline__ void clear(int v) const { w[v] = kDistMask; }
-    __device__ __forceinline__ int offer(int v, unsigned long long nd, double sg) const {
+    using Seen = unsigned long long;  // ... its whole word, which the first compare-and-swap expects
+    __device__ __forceinline__ Seen look(int v) const { return w[v]; }
+    static __device__ __forceinline__ unsigned long long dist_of(Seen x) { return x & kDistMask; }
+    __device__ __forceinline__ int offer(int v, unsigned long long nd, double sg, Seen cur) const {
         if (nd >= kDistMask) return kOfferWide;
         const unsigned long long si = (unsigned long long)sg;  // an integer below 2^40
-        unsigned long long cur = w[v];
         for (int it = 0; it < kCasTries; ++it) {
             const unsigned long long cd = cur & kDistMask;
             if (nd > cd) return kOfferNone;
@@ -210,44 +226,75 @@ struct NarrowPairs {
     }
 };
 
-// Offers out-arcs a, a + step, ... < ae of a vertex settled at distance d
-// with path count sg: lowers a head's distance (and queues it) or adds sg to
-// its count when the candidate ties. With tb (Eq. 4 launches), an offer that
-// took effect also sets its arc's bit: every tight arc gets one (its offer
+// Arcs of a group of settled vertices, staged by one warp: the arcs of lane
+// i's vertex end at incl[i] in the group's order; arc k of the group sits at
+// off[its vertex] + k.
+struct WarpArcs {
+    int incl[32];
+    long long off[32];
+    double sg[32];  // path counts of the vertices
+};
+
+// Offers the group's arcs, kLanesBatch per lane in flight, of vertices settled
+// at distance d: an offer lowers a head's distance (and queues it) or adds the
+// tail's path count when the candidate ties. With tb (Eq. 4 launches), an offer
+// that took effect also sets its arc's bit: every tight arc gets one (its offer
 // of the final distance always takes effect), and arcs whose offer a shorter
-// path replaced keep a stale bit that the backward's check drops. Returns 0,
-// or the device error to raise (a pair that kept changing, a count or
-// distance the narrow layout cannot hold).
-template <class PairT>
-__device__ __forceinline__ int src_relax(const TravParams &p, const PairT &P, uint32_t *bk, uint32_t *s_cnt,
-                                         uint32_t *tb, int64_t bcap, int R, unsigned long long d, double sg,
-                                         long long a, long long ae, int step, unsigned long long &adds) {
+// path replaced keep a stale bit that the backward's check drops. Returns 0, or
+// the device error to raise (a pair that kept changing, a count or distance the
+// narrow layout cannot hold).
+template <class PairT, bool kBits>
+__device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, uint32_t *bk, uint32_t *s_cnt,
+                                          const uint32_t *s_done, uint32_t *tb, int64_t bcap, int R,
+                                          unsigned long long d, const WarpArcs &wa, int total,
+                                          unsigned long long &adds) {
+    const int lane = threadIdx.x & 31;
     int err = 0;
-    for (; a < ae; a += kLanesBatch * step) {
+    for (int base = lane; base < total; base += 32 * kLanesBatch) {
         int y[kLanesBatch];
-        unsigned long long nd[kLanesBatch], cd[kLanesBatch];
+        uint32_t w[kLanesBatch];
+        unsigned vs = 0;  // the arcs' vertices, 5 bits each
 #pragma unroll
         for (int j = 0; j < kLanesBatch; ++j) {
-            const long long aj = a + (long long)j * step;
-            y[j] = aj < ae ? __ldg(p.col + aj) : -1;
-            nd[j] = aj < ae ? d + __ldg(p.wt + aj) : 0ull;
+            const int i = base + 32 * j;
+            int v = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (wa.incl[v + o - 1] <= i) v += o;
+            vs |= (unsigned)v << (5 * j);
+            y[j] = -1;
+            if (i < total) {
+                const long long a = wa.off[v] + i;
+                y[j] = __ldg(p.col + a);
+                w[j] = __ldg(p.wt + a);
+            }
         }
-        // the heads' distances first; the compare-and-swap only for the few
-        // candidates that lower or tie
+        if (kBits) {
 #pragma unroll
-        for (int j = 0; j < kLanesBatch; ++j) cd[j] = y[j] >= 0 ? P.dist(y[j]) : 0ull;
+            for (int j = 0; j < kLanesBatch; ++j)
+                if (y[j] >= 0 && ((s_done[y[j] >> 5] >> (y[j] & 31)) & 1u)) y[j] = -1;
+        }
+        // the heads first; the compare-and-swap only for the few candidates
+        // that lower or tie
+        typename PairT::Seen cur[kLanesBatch];
+#pragma unroll
+        for (int j = 0; j < kLanesBatch; ++j)
+            if (y[j] >= 0) cur[j] = P.look(y[j]);
 #pragma unroll
         for (int j = 0; j < kLanesBatch; ++j) {
-            if (y[j] < 0 || nd[j] > cd[j]) continue;
-            const int r = P.offer(y[j], nd[j], sg);
+            if (y[j] < 0) continue;
+            const unsigned long long nd = d + w[j];
+            if (nd > PairT::dist_of(cur[j])) continue;
+            const int v = (int)(vs >> (5 * j)) & 31;
+            const int r = P.offer(y[j], nd, wa.sg[v], cur[j]);
             if (r > 0) {
                 adds += 1;
                 if (tb) {
-                    const long long aj = a + (long long)j * step;
-                    atomicOr(tb + (aj >> 5), 1u << (aj & 31));
+                    const long long a = wa.off[v] + base + 32 * j;
+                    atomicOr(tb + (a >> 5), 1u << (a & 31));
                 }
                 if (r == kOfferLower) {
-                    const int slot = (int)(nd[j] & (unsigned long long)(R - 1));
+                    const int slot = (int)(nd & (unsigned long long)(R - 1));
                     const uint32_t pos = atomicAdd(&s_cnt[slot], 1u);
                     bk[(size_t)slot * (size_t)bcap + (pos & (uint32_t)(bcap - 1))] = (uint32_t)y[j];
                 }
@@ -261,37 +308,36 @@ __device__ __forceinline__ int src_relax(const TravParams &p, const PairT &P, ui
     return err;
 }
 
-// Sum of c(y) over the tight out-arcs (y at distance d + w(v, y)) among a,
-// a + step, ... < ae of a vertex at distance d. Only arcs whose bit the
-// forward set can be tight; the others are skipped without reading their
-// head.
+// Sum of c(y) over the tight out-arcs (y at distance d + w(v, y)) among arcs
+// [a, ae) of a vertex at distance d, this lane's share: the words rl, rl + lpp,
+// ... of the row's arc bits. Only arcs whose bit the forward set can be tight.
 __device__ __forceinline__ double src_pull_c(const TravParams &p, const DistSig *ds, const uint32_t *tb,
-                                             unsigned long long d, long long a, long long ae, int step) {
+                                             unsigned long long d, long long a, long long ae, int rl, int lpp) {
     double acc = 0.0;
-    for (; a < ae; a += kLanesBatch * step) {
-        int y[kLanesBatch];
-        unsigned long long want[kLanesBatch];
-        bool ok[kLanesBatch];
+    if (ae <= a) return acc;
+    const long long w0 = a >> 5, w1 = (ae - 1) >> 5;
+    for (long long w = w0 + rl; w <= w1; w += lpp) {
+        uint32_t bits = tb[w];
+        if (w == w0) bits &= ~0u << (a & 31);
+        if (w == w1) bits &= ~0u >> (31 - ((ae - 1) & 31));
+        while (bits) {
+            bool ok[kPullBatch];
+            unsigned long long want[kPullBatch];
+            DistSig v[kPullBatch];
 #pragma unroll
-        for (int j = 0; j < kLanesBatch; ++j) {
-            const long long aj = a + (long long)j * step;
-            ok[j] = aj < ae && ((tb[aj >> 5] >> (aj & 31)) & 1u);
-            y[j] = ok[j] ? __ldg(p.col + aj) : 0;
-            want[j] = ok[j] ? d + __ldg(p.wt + aj) : 0ull;
-        }
-        DistSig v[kLanesBatch];
-#pragma unroll
-        for (int j = 0; j < kLanesBatch; ++j) {
-            if (ok[j]) {
-                v[j] = ds[y[j]];
-            } else {
-                v[j].d = ~0ull;
-                v[j].s = 0.0;
+            for (int j = 0; j < kPullBatch; ++j) {
+                ok[j] = bits != 0u;
+                const long long aj = 32 * w + (ok[j] ? __ffs(bits) - 1 : 0);
+                bits &= bits - 1u;
+                if (ok[j]) {
+                    want[j] = d + __ldg(p.wt + aj);
+                    v[j] = ds[__ldg(p.col + aj)];
+                }
             }
-        }
 #pragma unroll
-        for (int j = 0; j < kLanesBatch; ++j)
-            if (ok[j] && v[j].d == want[j]) acc += v[j].s;
+            for (int j = 0; j < kPullBatch; ++j)
+                if (ok[j] && v[j].d == want[j]) acc += v[j].s;
+        }
     }
     return acc;
 }
@@ -334,16 +380,17 @@ __device__ __forceinline__ void src_finalize(const TravParams &p, DistSig *ds, u
     }
 }
 
-template <class PairT>
+template <class PairT, bool kBits>
 __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcParams q) {
-    extern __shared__ uint32_t s_ring[];  // [2 * R]: queued, then consumed, per slot
+    extern __shared__ __align__(16) unsigned char s_src[];  // WarpArcs per warp, ring counters, settled bits
     __shared__ int32_t s_ql[64];          // level at which query vertex q settled for this source
     __shared__ double s_dep[64];
     __shared__ double s_msum[64];         // several query vertices: per-column scan sums
     __shared__ unsigned long long s_cd[64];  // ... d(s, croot[c])
     __shared__ double s_red[32];
     __shared__ long long s_i;
-    __shared__ int s_k, s_nh, s_err, s_flag, s_stop;
+    __shared__ int s_k, s_nh, s_err, s_flag, s_stop, s_group;
+    const long long pack_max = (long long)kPackRows * p.wshort;
     __shared__ int s_nch[2];  // chunks of the current level, by level parity
     __shared__ unsigned long long s_t0;
 
@@ -353,8 +400,13 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
     const int R = q.ring;
     const int64_t bcap = q.bcap;
     const int CH = p.chunk_arcs;
+    const int CHB = max(CH, 1024);  // backward chunks: a word of arc bits per lane
+    WarpArcs &wa = reinterpret_cast<WarpArcs *>(s_src)[threadIdx.x >> 5];
+    uint32_t *s_ring = reinterpret_cast<uint32_t *>(s_src + sizeof(WarpArcs) * (blockDim.x >> 5));  // [2 * R]: queued, then consumed, per slot
     uint32_t *s_cnt = s_ring;
     uint32_t *s_base = s_ring + R;
+    uint32_t *s_done = s_ring + 2 * R;  // [(n + 31) / 32]
+    const int done_words = kBits ? (int)((q.n + 31) / 32) : 0;
     const size_t boff = (size_t)blockIdx.x * (size_t)q.n;
     DistSig *ds = q.ds + boff;  // wide pairs (Eq. 4 reads and writes them directly)
     PairT P;
@@ -395,7 +447,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             t_mark = t;
             s_t0 = t;
         }
-        for (int k = tid; k < 2 * R; k += bd) s_ring[k] = 0u;
+        for (int k = tid; k < 2 * R + done_words; k += bd) s_ring[k] = 0u;
         for (int k = tid; k < 64; k += bd) {
             s_ql[k] = -1;
             s_dep[k] = 0.0;
@@ -419,7 +471,10 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
         int seg = 0, nh = 0;
         bool first = true;
         for (;;) {
-            if (tid == 0) s_k = R;
+            if (tid == 0) {
+                s_k = R;
+                s_group = 0;
+            }
             __syncthreads();
             for (int k = tid + (first ? 0 : 1); k < R; k += bd) {
                 const int sl = (int)((d + (unsigned long long)k) & (unsigned long long)(R - 1));
@@ -445,67 +500,94 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                 ldist[seg] = d;
             }
             int *nchp = &s_nch[seg & 1];
-            // step 1: the slot's vertices; short rows finish here
+            // step 1: the slot's vertices, in groups that the warps draw; their
+            // rows finish here unless they are long
             {
-                const int lpp = lanes_per_vertex((long long)cnt, bd);
-                const int per = 32 / lpp, sub = lane / lpp, rl = lane % lpp;
-                const bool lead = rl == 0;
-                const long long ngroups = ((long long)cnt + per - 1) / per;
+                // one group per warp on a thin level, about two on others
+                const unsigned warps = (unsigned)nwarps;
+                const unsigned share = cnt <= 16 * warps ? (cnt + warps - 1) / warps : (cnt + 2 * warps - 1) / (2 * warps);
+                const int gsize = (int)min(32u, share);
                 const uint32_t *bks = bk + (size_t)slot * (size_t)bcap;
-                for (long long gi = warp; gi < ngroups; gi += nwarps) {
-                    const long long ii = gi * per + sub;
-                    int x = 0;
+                for (;;) {
+                    int g0 = 0;
+                    if (lane == 0) g0 = atomicAdd(&s_group, gsize);
+                    g0 = __shfl_sync(kFull, g0, 0);
+                    if ((uint32_t)g0 >= cnt) break;
+                    // all that a queued vertex needs, in one round of loads
+                    int x = 0, seen = 0;
                     unsigned long long xd = PairT::kUnreached;
                     double xs = 0.0;
-                    if (ii < (long long)cnt) {
-                        x = (int)bks[(b0 + (uint32_t)ii) & (uint32_t)(bcap - 1)];
+                    long long rb = 0, re = 0;
+                    uint64_t qm = 0ull;
+                    if (lane < gsize && (uint32_t)(g0 + lane) < cnt) {
+                        x = (int)bks[(b0 + (uint32_t)(g0 + lane)) & (uint32_t)(bcap - 1)];
                         P.get(x, xd, xs);
+                        rb = __ldg(p.off + x);
+                        re = __ldg(p.off + x + 1);
+                        seen = *(volatile const int32_t *)(p.tag + x);
+                        qm = __ldg(p.qmask + x);
                     }
                     const bool ok = xd == d;
-                    const unsigned am = __ballot_sync(kFull, ok && lead);
+                    const unsigned am = __ballot_sync(kFull, ok);
                     if (am == 0u) continue;
                     int eb = 0;
                     if (lane == 0) eb = atomicAdd(&s_nh, __popc(am));
                     eb = __shfl_sync(kFull, eb, 0);
-                    const int e = eb + __popc(am & ((1u << (sub * lpp)) - 1u));
-                    long long rb = 0, re = 0;
+                    int len = 0;
                     if (ok) {
-                        rb = __ldg(p.off + x);
-                        re = __ldg(p.off + x + 1);
-                    }
-                    if (ok && lead) {
-                        hv[e] = x;
+                        const long long deg = re - rb;
+                        hv[eb + __popc(am & ((1u << lane) - 1u))] = x;
+                        if (kBits) atomicOr(&s_done[x >> 5], 1u << (x & 31));
                         st.reached += 1;
-                        st.edges += (unsigned long long)(re - rb);
+                        st.edges += (unsigned long long)deg;
                         if (xs >= kSrcTwo53) s_flag = 1;
-                        if (*(volatile const int32_t *)(p.tag + x) == -1 && atomicCAS(&p.tag[x], -1, 0) == -1) {
+                        if (seen == -1 && atomicCAS(&p.tag[x], -1, 0) == -1) {
                             st.vb += 1;
-                            st.eb += (unsigned long long)(re - rb);
+                            st.eb += (unsigned long long)deg;
                         }
-                        uint64_t y = __ldg(p.qmask + x) & need;
+                        uint64_t y = qm & need;
                         while (y) {
                             const int qq = __ffsll((long long)y) - 1;
                             y &= y - 1;
                             s_ql[qq] = seg;
                         }
-                    }
-                    if (ok && re - rb <= p.wshort) {
-                        if (lead) st.arcs += (unsigned long long)(re - rb);
-                        const int er = src_relax(p, P, bk, s_cnt, tb, bcap, R, d, xs, rb + rl, re, lpp, st.tight);
-                        if (er) {
-                            s_err = 1;
-                            set_err(p.ctr, er);
-                        }
-                    } else if (ok && lead) {
-                        const int nout = (int)((re - rb + CH - 1) / CH);
-                        const int c0 = atomicAdd(nchp, nout);
-                        if ((int64_t)c0 + nout > q.chcap) {
-                            s_err = 1;
-                            set_err(p.ctr, kDevChunkOverflow);
+                        if (deg <= pack_max) {
+                            len = (int)deg;
+                            st.arcs += (unsigned long long)deg;
                         } else {
-                            src_store_chunks(chs, c0, x, e, 0, rb, re, nout, CH);
+                            const int nout = (int)((deg + CH - 1) / CH);
+                            const int c0 = atomicAdd(nchp, nout);
+                            if ((int64_t)c0 + nout > q.chcap) {
+                                s_err = 1;
+                                set_err(p.ctr, kDevChunkOverflow);
+                            } else {
+                                // the chunks carry the path count in place of entry and index
+                                for (int k = 0; k < nout; ++k) {
+                                    const long long a0 = rb + (long long)k * CH;
+                                    store_chunk(&chs[c0 + k], x, __double2loint(xs), __double2hiint(xs), nout, a0,
+                                                (int)(min(rb + deg, a0 + CH) - a0));
+                                }
+                            }
                         }
                     }
+                    // the group's arcs, packed onto the lanes
+                    int incl = len;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int z = __shfl_up_sync(kFull, incl, o);
+                        if (lane >= o) incl += z;
+                    }
+                    wa.incl[lane] = incl;
+                    wa.off[lane] = rb - (incl - len);
+                    wa.sg[lane] = xs;
+                    const int total = __shfl_sync(kFull, incl, 31);
+                    __syncwarp();
+                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, total, st.tight);
+                    if (er) {
+                        s_err = 1;
+                        set_err(p.ctr, er);
+                    }
+                    __syncwarp();
                 }
             }
             __syncthreads();
@@ -523,14 +605,19 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             if (nch > 0) {
                 for (int c = warp; c < nch; c += nwarps) {
                     const Chunk ch = load_chunk(&chs[c]);
-                    unsigned long long cdv;
-                    double sg;
-                    P.get(ch.v, cdv, sg);
-                    const int er = src_relax(p, P, bk, s_cnt, tb, bcap, R, d, sg, ch.a0 + lane, ch.a0 + ch.na, 32, st.tight);
+                    const double xs = __hiloint2double(ch.k, ch.e);
+                    wa.incl[lane] = ch.na;
+                    if (lane == 0) {
+                        wa.off[0] = ch.a0;
+                        wa.sg[0] = xs;
+                    }
+                    __syncwarp();
+                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, ch.na, st.tight);
                     if (er) {
                         s_err = 1;
                         set_err(p.ctr, er);
                     }
+                    __syncwarp();
                     if (lane < ch.na) st.arcs += (unsigned long long)((ch.na - lane + 31) / 32);
                 }
                 __syncthreads();
@@ -661,21 +748,21 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                         rb = __ldg(p.off + v);
                         re = __ldg(p.off + v + 1);
                     }
-                    const bool shortrow = ok && re - rb <= p.wshort;
+                    const bool shortrow = ok && re - rb <= pack_max;
                     double acc = 0.0;
-                    if (shortrow) acc = src_pull_c(p, ds, tb, dk, rb + rl, re, lpp);
+                    if (shortrow) acc = src_pull_c(p, ds, tb, dk, rb, re, rl, lpp);
                     acc = sum_lanes(acc, lpp);
                     if (shortrow && lead) {
                         src_finalize(p, ds, need, s_dep, v, acc);
                         st.arcs += (unsigned long long)(re - rb);
                     } else if (ok && !shortrow && lead) {
-                        const int nout = (int)((re - rb + CH - 1) / CH);
+                        const int nout = (int)((re - rb + CHB - 1) / CHB);
                         const int c0 = atomicAdd(nchp, nout);
                         if ((int64_t)c0 + nout > q.chcap) {
                             s_err = 1;
                             set_err(p.ctr, kDevChunkOverflow);
                         } else {
-                            src_store_chunks(chs, c0, v, (int)(e0 + ii), 0, rb, re, nout, CH);
+                            src_store_chunks(chs, c0, v, (int)(e0 + ii), 0, rb, re, nout, CHB);
                         }
                     }
                 }
@@ -692,7 +779,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                 if (nch > 0) {
                     for (int c = warp; c < nch; c += nwarps) {
                         const Chunk ch = load_chunk(&chs[c]);
-                        const double v = sum_warp(src_pull_c(p, ds, tb, dk, ch.a0 + lane, ch.a0 + ch.na, 32));
+                        const double v = sum_warp(src_pull_c(p, ds, tb, dk, ch.a0, ch.a0 + ch.na, lane, 32));
                         if (lane == 0) part[c] = v;
                         if (lane < ch.na) st.arcs += (unsigned long long)((ch.na - lane + 31) / 32);
                     }
@@ -786,6 +873,17 @@ __global__ void wsrc_tile_sums(TravParams p, const double *sdep, const uint32_t 
         }
     }
 }
+
+// Threads per block. A distance level is a chain of about five dependent loads
+// and two or three block barriers whatever it holds, so small blocks, with more
+// sources in flight per SM, win while the state of all of them (8 or 16 bytes
+// per vertex and source) stays near L2; with larger graphs it is pushed out to
+// DRAM and fewer, wider blocks win. Weights 1..255 (2,000 draws or all sources),
+// 1024 / 512 / 256 / 128 threads: n = 5,000 8.9 / 5.0 / 3.8 / 4.3 ms, 32,768
+// 26.5 / 17.9 / 14.7 / 20.3, 65,536 82.7 / 63.7 / 57.0 / 75.2, 131,072 31.5 /
+// 27.9 / 32.0 / 52.0, 262,144 55.2 / 52.5 / 68.5 / 136, 524,288 104 / 110 / 260
+// / 334, R-MAT 20 280 / 411 / 735 / 1402.
+int src_threads(int64_t n) { return n <= 96 * 1024 ? 256 : n <= 384 * 1024 ? 512 : kSrcThreads; }
 
 // Bytes of per-block state for a graph of n vertices.
 size_t src_block_bytes(int64_t n, int64_t m, int R, int64_t bcap, int64_t maxlev, int64_t chcap) {
@@ -894,24 +992,31 @@ bool src_kernel_applies(const bc_graph *g, const TravParams &p) {
 bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsigned long long *edges_out) {
     bcd_workspace &ws = g->ws;
     BCD_TRY(ensure_weighted_state(g));  // ring size, tag array
-    const int threads = kSrcThreads;
+    const int threads = src_threads(g->n);
     const int S = 64 * W;
     const int64_t nsrc = p.ntiles * S;
     const int R = ws.ring;
-    const size_t smem = sizeof(uint32_t) * 2 * (size_t)R;
+    // the settled bits join the staging and counters in shared memory while they fit
+    const size_t ring = sizeof(WarpArcs) * (size_t)(threads / 32) + sizeof(uint32_t) * 2 * (size_t)R;
+    const size_t done = sizeof(uint32_t) * (((size_t)g->n + 31) / 32);
+    const bool bits = ring + done <= kSrcDynSmem;
+    const size_t smem = ring + (bits ? done : 0);
+    const void *wide = bits ? (const void *)wsrc_kernel<WidePairs, true> : (const void *)wsrc_kernel<WidePairs, false>;
+    const void *narrow = bits ? (const void *)wsrc_kernel<NarrowPairs, true> : (const void *)wsrc_kernel<NarrowPairs, false>;
     int per_sm = 0, per_sm_n = 0;
-    BCD_CUDA(cudaFuncSetAttribute(wsrc_kernel<WidePairs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    BCD_CUDA(cudaFuncSetAttribute(wsrc_kernel<NarrowPairs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wsrc_kernel<WidePairs>, threads, smem));
-    BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_n, wsrc_kernel<NarrowPairs>, threads, smem));
+    BCD_CUDA(cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BCD_CUDA(cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide, threads, smem));
+    BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_n, narrow, threads, smem));
     per_sm = std::min(per_sm, per_sm_n);
     if (per_sm < 1) return set_error(BC_E_INTERNAL, "weighted source kernel cannot be resident");
     if (ws.sbcap == 0) {
         // queued vertices of one distance of one source: a few times the
         // average vertices per distance value, and at least 2^21 entries
-        // over the whole ring (8 MB); grown on overflow
+        // over the whole ring (8 MB), or 32 per vertex; grown on overflow
+        const int64_t whole = std::min<int64_t>((int64_t)1 << 21, 32 * (int64_t)g->n);
         int64_t b = 64;
-        while ((b < 4 * (int64_t)g->n / R || b * R < ((int64_t)1 << 21)) && b < ((int64_t)1 << 30)) b *= 2;
+        while ((b < 4 * (int64_t)g->n / R || b * R < whole) && b < ((int64_t)1 << 30)) b *= 2;
         ws.sbcap = b;
         ws.schcap = 16384;
         ws.smaxlev = 8192;
@@ -978,13 +1083,11 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         const bool timed = cudaEventCreate(&ev0) == cudaSuccess && cudaEventCreate(&ev1) == cudaSuccess;
         if (timed) cudaEventRecord(ev0, g->stream);
-        if (layout == 2)
-            wsrc_kernel<NarrowPairs><<<(unsigned)ws.sblocks, (unsigned)threads, smem, g->stream>>>(p, q);
-        else
-            wsrc_kernel<WidePairs><<<(unsigned)ws.sblocks, (unsigned)threads, smem, g->stream>>>(p, q);
+        void *args[] = {(void *)&p, (void *)&q};
+        const cudaError_t le = cudaLaunchKernel(layout == 2 ? narrow : wide, dim3((unsigned)ws.sblocks),
+                                                dim3((unsigned)threads), args, smem, g->stream);
         g->launches += 1;
         g->last_grid = ws.sblocks;
-        const cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) {
             if (timed) {
                 cudaEventDestroy(ev0);
