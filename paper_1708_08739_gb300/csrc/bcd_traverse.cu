@@ -840,17 +840,26 @@ __device__ __noinline__ void pull_level(int L, const uint64_t *s_valid, long lon
     if (over) set_err(p.ctr, kDevWide);
 }
 
+// 1 / sigma. The chip's fp64 units are few (a warp instruction holds an SM's
+// for 16 cycles, so the dozen of a division cost more than the rest of a
+// step): counts up to kInverses, nearly all of them, are looked up.
+constexpr int kInverses = 2048;
+__device__ __forceinline__ double inverse_of(const double *s_inv, uint32_t x) {
+    return x < (uint32_t)kInverses ? s_inv[x] : 1.0 / (double)x;
+}
+__device__ __forceinline__ double inverse_of(const double *s_inv, double x) { return 1.0 / x; }
+
 // Eq. 4, push form, from level L into level L - 1: each entry w of level L
-// sends c_s(w) = (1 + delta_s(w)) / sigma_s(w), with delta_s(w) =
-// sigma_s(w) * acc_s(w) complete (level L + 1 pushed into it in the previous
-// step), back along its in-arcs (v, w) that are tight for a source s still
+// sends c_s(w) = (1 + delta_s(w)) / sigma_s(w) = 1 / sigma_s(w) + acc_s(w)
+// (delta_s(w) = sigma_s(w) * acc_s(w), complete: level L + 1 pushed into it in
+// the previous step) back along its in-arcs (v, w) that are tight for a source s still
 // active at L - 1 (v at level L - 1 for s), adding it to acc_s(v) with fp64
 // atomic adds. c is formed on the fly from the sigma and acc slabs, which this
 // step only reads for level-L pairs. The in-arc chunks of level L were cut in
 // the forward pass. Lane l holds sources l + 32 i; two tight tails per step.
 template <int W, typename T>
 __device__ void push_level(const TravParams &p, int L, long long ics, long long ccnt, const uint64_t *s_act,
-                           long long nwarps) {
+                           const double *s_inv, long long nwarps) {
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
     const int lane = threadIdx.x & 31;
@@ -869,15 +878,16 @@ __device__ void push_level(const TravParams &p, int L, long long ics, long long 
 #pragma unroll
         for (int k = 0; k < W; ++k) F[k] = p.hm[(size_t)ch.e * W + k] & s_act[k];
         const T *sigma = reinterpret_cast<const T *>(p.sigma);
-        double sw[PL], aw[PL], cw[PL];
+        double cw[PL];
+        T sw[PL];
 #pragma unroll
         for (int ii = 0; ii < PL; ++ii) {
-            sw[ii] = (double)sigma[(size_t)w * S + lane + 32 * ii];
-            aw[ii] = p.acc[(size_t)w * S + lane + 32 * ii];
+            const bool in = mask_bit<W>(F, lane + 32 * ii);
+            sw[ii] = in ? sigma[(size_t)w * S + lane + 32 * ii] : T(1);
+            cw[ii] = in ? p.acc[(size_t)w * S + lane + 32 * ii] : 0.0;
         }
 #pragma unroll
-        for (int ii = 0; ii < PL; ++ii)
-            cw[ii] = mask_bit<W>(F, lane + 32 * ii) ? (1.0 + sw[ii] * aw[ii]) / sw[ii] : 0.0;
+        for (int ii = 0; ii < PL; ++ii) cw[ii] += inverse_of(s_inv, sw[ii]);
         for (int base = 0; base < na; base += 32) {
             const bool valid = base + lane < na;
             const int v = vnext;
@@ -1292,6 +1302,9 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
     __shared__ uint64_t s_active_next[W];
     __shared__ uint64_t s_valid[W];  // the tile's occupied source slots
     __shared__ int32_t s_lstop;
+    __shared__ double s_inv[MODE == kModeSpd ? kInverses : 1];  // Eq. 4: 1 / k
+    if (MODE == kModeSpd)
+        for (int i = threadIdx.x; i < kInverses; i += blockDim.x) s_inv[i] = 1.0 / (double)max(i, 1);
     const bool timer = team == 0 && leader;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
     unsigned long long ns_fwd = 0, ns_bwd = 0, ns_other = 0;
@@ -1483,7 +1496,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                     if (more) {
                         const long long ics = p.lev_icstart[Lb];
                         const long long ic = (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + Lb]);
-                        push_level<W, T>(p, Lb, ics, ic, s_active_next, nwarps);
+                        push_level<W, T>(p, Lb, ics, ic, s_active_next, s_inv, nwarps);
                     }
                     if (!team_barrier(p, gen)) return;
                 }

@@ -151,6 +151,8 @@ struct WidePairs {
     static constexpr unsigned long long kUnreached = ~0ull;
     DistSig *ds;
     __device__ __forceinline__ unsigned long long dist(int v) const { return ds[v].d; }
+    using Count = double;
+    static __device__ __forceinline__ bool two53(double s) { return s >= kSrcTwo53; }
     __device__ __forceinline__ void get(int v, unsigned long long &d, double &sg) const {
         const DistSig x = ds[v];
         d = x.d;
@@ -198,19 +200,20 @@ struct NarrowPairs {
     static constexpr unsigned long long kSigLimit = 1ull << 40;
     unsigned long long *w;
     __device__ __forceinline__ unsigned long long dist(int v) const { return w[v] & kDistMask; }
-    __device__ __forceinline__ void get(int v, unsigned long long &d, double &sg) const {
+    using Count = unsigned long long;  // converted to fp64 only where a dependency needs it
+    static __device__ __forceinline__ bool two53(unsigned long long) { return false; }
+    __device__ __forceinline__ void get(int v, unsigned long long &d, unsigned long long &sg) const {
         const unsigned long long x = w[v];
         d = x & kDistMask;
-        sg = (double)(x >> 24);
+        sg = x >> 24;
     }
     __device__ __forceinline__ void seed(int v) const { w[v] = 1ull << 24; }
     __device__ __forceinline__ void clear(int v) const { w[v] = kDistMask; }
     using Seen = unsigned long long;  // ... its whole word, which the first compare-and-swap expects
     __device__ __forceinline__ Seen look(int v) const { return w[v]; }
     static __device__ __forceinline__ unsigned long long dist_of(Seen x) { return x & kDistMask; }
-    __device__ __forceinline__ int offer(int v, unsigned long long nd, double sg, Seen cur) const {
+    __device__ __forceinline__ int offer(int v, unsigned long long nd, unsigned long long si, Seen cur) const {
         if (nd >= kDistMask) return kOfferWide;
-        const unsigned long long si = (unsigned long long)sg;  // an integer below 2^40
         for (int it = 0; it < kCasTries; ++it) {
             const unsigned long long cd = cur & kDistMask;
             if (nd > cd) return kOfferNone;
@@ -226,13 +229,22 @@ struct NarrowPairs {
     }
 };
 
+__device__ __forceinline__ unsigned long long to_bits(unsigned long long x) { return x; }
+__device__ __forceinline__ unsigned long long to_bits(double x) { return (unsigned long long)__double_as_longlong(x); }
+template <class C>
+__device__ __forceinline__ C from_bits(unsigned long long x);
+template <>
+__device__ __forceinline__ unsigned long long from_bits<unsigned long long>(unsigned long long x) { return x; }
+template <>
+__device__ __forceinline__ double from_bits<double>(unsigned long long x) { return __longlong_as_double((long long)x); }
+
 // Arcs of a group of settled vertices, staged by one warp: the arcs of lane
 // i's vertex end at incl[i] in the group's order; arc k of the group sits at
 // off[its vertex] + k.
 struct WarpArcs {
     int incl[32];
     long long off[32];
-    double sg[32];  // path counts of the vertices
+    unsigned long long sg[32];  // path counts of the vertices (integers or the bits of a double)
 };
 
 // Offers the group's arcs, kLanesBatch per lane in flight, of vertices settled
@@ -286,7 +298,7 @@ __device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, u
             const unsigned long long nd = d + w[j];
             if (nd > PairT::dist_of(cur[j])) continue;
             const int v = (int)(vs >> (5 * j)) & 31;
-            const int r = P.offer(y[j], nd, wa.sg[v], cur[j]);
+            const int r = P.offer(y[j], nd, from_bits<typename PairT::Count>(wa.sg[v]), cur[j]);
             if (r > 0) {
                 adds += 1;
                 if (tb) {
@@ -366,17 +378,17 @@ __device__ __forceinline__ void src_store_chunks(Chunk *chs, long long c0, int v
     }
 }
 
-// delta(v) = sigma(v) * acc; c(v) = (1 + delta(v)) / sigma(v) replaces sigma(v).
+// delta(v) = sigma(v) * acc; c(v) = (1 + delta(v)) / sigma(v) = 1 / sigma(v) +
+// acc replaces sigma(v).
 __device__ __forceinline__ void src_finalize(const TravParams &p, DistSig *ds, uint64_t need, double *s_dep, int v,
                                              double acc) {
     const double sv = ds[v].s;
-    const double dd = sv * acc;
-    ds[v].s = (1.0 + dd) / sv;
+    ds[v].s = 1.0 / sv + acc;
     uint64_t y = __ldg(p.qmask + v) & need;
     while (y) {
         const int q = __ffsll((long long)y) - 1;
         y &= y - 1;
-        s_dep[q] = dd;
+        s_dep[q] = sv * acc;
     }
 }
 
@@ -516,7 +528,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     // all that a queued vertex needs, in one round of loads
                     int x = 0, seen = 0;
                     unsigned long long xd = PairT::kUnreached;
-                    double xs = 0.0;
+                    typename PairT::Count xs = 0;
                     long long rb = 0, re = 0;
                     uint64_t qm = 0ull;
                     if (lane < gsize && (uint32_t)(g0 + lane) < cnt) {
@@ -540,7 +552,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                         if (kBits) atomicOr(&s_done[x >> 5], 1u << (x & 31));
                         st.reached += 1;
                         st.edges += (unsigned long long)deg;
-                        if (xs >= kSrcTwo53) s_flag = 1;
+                        if (PairT::two53(xs)) s_flag = 1;
                         if (seen == -1 && atomicCAS(&p.tag[x], -1, 0) == -1) {
                             st.vb += 1;
                             st.eb += (unsigned long long)deg;
@@ -564,7 +576,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                                 // the chunks carry the path count in place of entry and index
                                 for (int k = 0; k < nout; ++k) {
                                     const long long a0 = rb + (long long)k * CH;
-                                    store_chunk(&chs[c0 + k], x, __double2loint(xs), __double2hiint(xs), nout, a0,
+                                    store_chunk(&chs[c0 + k], x, (int)(unsigned)to_bits(xs), (int)(to_bits(xs) >> 32), nout, a0,
                                                 (int)(min(rb + deg, a0 + CH) - a0));
                                 }
                             }
@@ -579,7 +591,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     }
                     wa.incl[lane] = incl;
                     wa.off[lane] = rb - (incl - len);
-                    wa.sg[lane] = xs;
+                    wa.sg[lane] = to_bits(xs);
                     const int total = __shfl_sync(kFull, incl, 31);
                     __syncwarp();
                     const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, total, st.tight);
@@ -605,11 +617,10 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             if (nch > 0) {
                 for (int c = warp; c < nch; c += nwarps) {
                     const Chunk ch = load_chunk(&chs[c]);
-                    const double xs = __hiloint2double(ch.k, ch.e);
                     wa.incl[lane] = ch.na;
                     if (lane == 0) {
                         wa.off[0] = ch.a0;
-                        wa.sg[0] = xs;
+                        wa.sg[0] = ((unsigned long long)(unsigned)ch.k << 32) | (unsigned)ch.e;
                     }
                     __syncwarp();
                     const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, ch.na, st.tight);
@@ -644,7 +655,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             // d(s, r) + d(r, t) = d(s, t) of sigma_rt / sigma_st
             const int r = p.vroot;
             unsigned long long dsr;
-            double ssr;
+            typename PairT::Count ssr;
             P.get(r, dsr, ssr);
             double acc = 0.0;
             if (dsr != PairT::kUnreached && need) {
@@ -652,10 +663,10 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     const int t = hv[e];
                     const unsigned long long rd = p.rdist[t];
                     unsigned long long dt;
-                    double sst;
+                    typename PairT::Count sst;
                     P.get(t, dt, sst);
                     if (rd == 0ull || rd >= dt || dsr + rd != dt) continue;
-                    acc += p.rsig[t] / sst;
+                    acc += p.rsig[t] / (double)sst;
                     st.pairs += 1;
                 }
             }
@@ -665,7 +676,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             if (tid == 0) {
                 double sum = 0.0;
                 for (int w = 0; w < nwarps; ++w) sum += s_red[w];
-                const double dv = dsr != PairT::kUnreached ? ssr * sum : 0.0;
+                const double dv = dsr != PairT::kUnreached ? (double)ssr * sum : 0.0;
                 uint64_t y = need;
                 while (y) {
                     const int qq = __ffsll((long long)y) - 1;
@@ -690,7 +701,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             for (int e = tid; e < nh; e += bd) {
                 const int t = hv[e];
                 unsigned long long dt;
-                double sst;
+                typename PairT::Count sst;
                 P.get(t, dt, sst);
                 uint64_t y = cols;
                 while (y) {
@@ -700,7 +711,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     if (dc == PairT::kUnreached) continue;
                     const unsigned long long rd = p.rdistq[(size_t)t * wcols_stride(p.ncols) + c];
                     if (rd == 0ull || rd >= dt || dc + rd != dt) continue;
-                    atomicAdd(&s_msum[c], p.rsigq[(size_t)t * wcols_stride(p.ncols) + c] / sst);
+                    atomicAdd(&s_msum[c], p.rsigq[(size_t)t * wcols_stride(p.ncols) + c] / (double)sst);
                     st.pairs += 1;
                 }
             }
@@ -712,9 +723,9 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     y &= y - 1;
                     const int c = p.qcol[qq];
                     unsigned long long dcr;
-                    double scr;
+                    typename PairT::Count scr;
                     P.get(p.croot[c], dcr, scr);
-                    s_dep[qq] = s_cd[c] != PairT::kUnreached ? scr * s_msum[c] : 0.0;
+                    s_dep[qq] = s_cd[c] != PairT::kUnreached ? (double)scr * s_msum[c] : 0.0;
                 }
             }
         } else if constexpr (PairT::kWide) {
