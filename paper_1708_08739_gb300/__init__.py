@@ -291,13 +291,12 @@ def bc_graph_reverse(g: Graph):
 
 def bc_rv_compute(g: Graph, r: int) -> np.ndarray:
     """RV(r): ascending ids of the vertices with a path to r (r excluded)."""
+    # room for every vertex, so that one traversal both counts and lists
+    out = np.empty(g.n, dtype=np.int32)
     cnt = C.c_int64()
-    st = lib().bc_rv_compute(g.handle, int(r), None, 0, C.byref(cnt))
-    if st not in (BC_OK, BC_E_BUFFER_TOO_SMALL):
-        _check(st)
-    out = np.zeros(max(cnt.value, 1), dtype=np.int32)
     _check(lib().bc_rv_compute(g.handle, int(r), _ptr(out), out.shape[0], C.byref(cnt)))
-    return out[: cnt.value]
+    rv = out[: cnt.value]
+    return rv if 2 * cnt.value >= g.n else rv.copy()
 
 
 def _info_dict(info: bc_info) -> dict:
