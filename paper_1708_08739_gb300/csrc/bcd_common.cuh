@@ -45,7 +45,12 @@ struct Counters {
     unsigned long long vpairs;     // vertex scan: (t, s) pairs with the query vertex on a shortest s-t path
     unsigned long long pull_levels; // forward levels run bottom-up (pull over R(G))
     unsigned long long tiles_taken; // tiles handed out after each team's first
+    unsigned long long trial_pairs; // vertex scan on trial: the terms it would add
+    unsigned long long scan_skipped; // ... it was not made, the tile has no result
 };
+
+// Bytes from the counters to the teams' barrier words that follow them.
+constexpr size_t kCounterBytes = (sizeof(Counters) + 127) / 128 * 128;
 
 // Barrier words of one team of blocks (unweighted traversal), and its next
 // tile; a cache line each.
@@ -80,7 +85,21 @@ enum TravFlags : int32_t {
     kFlagNoReset = 2,      // leave the dense state dirty (probe export)
     kFlagFullBackward = 4, // backward down to level 0 for every source
     kFlagRootOut = 8,      // scan mode: write the level and sigma of source slot 0 to rlev / rsig
+    kFlagTrial = 16,       // scan mode, one tile: count the terms first, scan only when they are few enough
 };
+
+// Cost of one term of the vertex scan (a division and a shared-memory add,
+// with the lanes of a warp on one pair's sources) in units of one tight
+// (source, arc) pair of the Eq. 4 push (an fp64 reduction).
+constexpr unsigned long long kScanPairCost = 16;
+
+// Terms of a tile whose scan is not worth avoiding: it takes about as long as the
+// forward pass that the Eq. 4 pass would have to repeat.
+constexpr unsigned long long kScanAlways = 1ull << 23;
+
+__host__ __device__ inline bool scan_too_long(unsigned long long terms, unsigned long long tight) {
+    return terms > kScanAlways && terms * kScanPairCost > tight;
+}
 
 struct TravParams {
     int32_t n;
@@ -193,7 +212,6 @@ struct TravParams {
 struct bcd_workspace {
     int W = 0;           // mask words per tile (S = 64 W sources)
     int teams = 1;       // tiles whose state is held at once (unweighted): the arrays of state below hold that many
-    bcd::TeamBar *bar = nullptr;  // [teams]
     int64_t n = 0;
     int64_t m = 0;
     // dense state

@@ -327,7 +327,6 @@ void free_workspace(bc_graph *g) {
     bcd_workspace &ws = g->ws;
     g->root_cache.clear();  // the traversal tables go with the workspace
     g->root_cache_buf = nullptr;
-    dev_free(ws.bar);
     dev_free(ws.vs);
     dev_free(ws.tag);
     dev_free(ws.sigma);
@@ -430,7 +429,6 @@ static bc_status build_workspace(bc_graph *g, int W) {
     ws.vs_stride = g->weighted ? 4 : ((3 * W + 3) / 4) * 4;
     ws.teams = g->weighted ? 1 : teams_for(n, m, W);
     const size_t t = (size_t)ws.teams;
-    BCD_TRY(dev_alloc(&ws.bar, t));
     BCD_TRY(dev_alloc(&ws.vs, t * n * ws.vs_stride));
     BCD_TRY(dev_alloc(&ws.tag, t * n));
     // counts of unweighted graphs: 32 bits until a launch needs fp64; the
@@ -461,7 +459,7 @@ static bc_status build_workspace(bc_graph *g, int W) {
     BCD_TRY(dev_alloc(&ws.rtile, (size_t)64 * W));
     BCD_TRY(dev_alloc(&ws.qflags, 64));
     BCD_TRY(dev_alloc(&ws.srcflag, t * std::max(W, 4)));
-    BCD_TRY(dev_alloc(&ws.ctr, 1));
+    BCD_TRY(dev_alloc((char **)&ws.ctr, kCounterBytes + sizeof(TeamBar) * t));
     ws.scratch_len = scan_scratch_len(n) + 64;
     BCD_TRY(dev_alloc(&ws.scratch64, (size_t)ws.scratch_len + 256));
     BCD_TRY(dev_alloc(&ws.small, (size_t)kSmallWords));
@@ -743,12 +741,6 @@ static bool use_vertex_scan(const bc_graph *g, size_t nroots) {
     return g->accumulation >= 3 && nroots <= 64;
 }
 
-// Cost of one term of the vertex scan (a division and a shared-memory add,
-// with the lanes of a warp on one pair's sources) in units of one tight
-// (source, arc) pair of the Eq. 4 push (an fp64 reduction). Measured on the
-// R-MAT benchmark graphs: 13-20.
-constexpr unsigned long long kScanPairCost = 16;
-
 // Offsets in bcd_workspace::small of the column tables of a multi-vertex scan.
 constexpr int kSmallQcol = 1024;   // 64 int32: column of each query bit
 constexpr int kSmallCroot = 1056;  // 64 int32: vertex of each column
@@ -998,11 +990,11 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
     if (nrun > 0) {
         BCD_TRY(ensure_buf(&ws.tile_partial, &ws.tile_partial_cap, nrun * 64));
         // tiles [first, first + count) of this call's range, in scan or Eq. 4 mode
-        auto launch_tiles = [&](bool scan_mode, int64_t first, int64_t count) -> bc_status {
+        auto launch_tiles = [&](bool scan_mode, int64_t first, int64_t count, bool trial = false) -> bc_status {
             TravParams p;
             memset(&p, 0, sizeof(p));
             p.mode = scan_mode ? kModeScan : kModeSpd;
-            p.flags = 0;
+            p.flags = trial ? kFlagTrial : 0;
             if (scan_mode) {
                 p.rlev = ws.rlev;
                 p.rdist = ws.rdist;
@@ -1035,6 +1027,10 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
             int lv = 0;
             unsigned long long ed = 0;
             BCD_TRY(src_kernel_applies(g, p) ? run_src_traversal(g, W, p, &lv, &ed) : run_traversal(g, W, p, &lv, &ed));
+            if (g->last.scan_skipped) {  // not this tile's result: the Eq. 4 pass runs it again
+                tm.trav += g->last_ms_launch;
+                return BC_OK;
+            }
             levels = std::max(levels, lv);
             edges += ed;
             tm.fwd += g->last_ns_fwd * 1e-6;
@@ -1055,18 +1051,26 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
             return BC_OK;
         };
         std::vector<uint32_t> cal_flags(64, 0);
-        if (multi && g->accumulation == 4 && nrun > 1) {
+        if (multi && g->accumulation == 4 && (nrun > 1 || !g->weighted)) {
             // choose the backward on the group's first tile: the scan's terms
             // (a division and a shared-memory add each) against the push's
             // tight (source, arc) pairs (an fp64 reduction each), at the
-            // measured cost ratio of about 16
-            BCD_TRY(launch_tiles(true, 0, 1));
-            BCD_CUDA(cudaMemcpyAsync(cal_flags.data(), ws.qflags, 64 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-            BCD_CUDA(cudaStreamSynchronize(s));
-            const bool scan_rest = g->last.vpairs * kScanPairCost <= g->last.tight;
-            tm.scan_tiles += 1;
-            BCD_TRY(launch_tiles(scan_rest, 1, nrun - 1));
-            if (scan_rest) tm.scan_tiles += nrun - 1;
+            // measured cost ratio of about 16. Unweighted: the terms are
+            // counted before any is added, and a tile with too many of them is
+            // left to the push (R-MAT 20 with hubs among the query vertices: 373
+            // million terms took 70 ms on the one tile, counting them and
+            // repeating its forward pass 5 ms).
+            BCD_TRY(launch_tiles(true, 0, 1, !g->weighted));
+            if (g->last.scan_skipped) {
+                BCD_TRY(launch_tiles(false, 0, nrun));
+            } else {
+                BCD_CUDA(cudaMemcpyAsync(cal_flags.data(), ws.qflags, 64 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+                BCD_CUDA(cudaStreamSynchronize(s));
+                const bool scan_rest = g->last.vpairs * kScanPairCost <= g->last.tight;
+                tm.scan_tiles += 1;
+                if (nrun > 1) BCD_TRY(launch_tiles(scan_rest, 1, nrun - 1));
+                if (scan_rest) tm.scan_tiles += nrun - 1;
+            }
         } else {
             BCD_TRY(launch_tiles(scan, 0, nrun));
             if (scan) tm.scan_tiles += nrun;
@@ -1261,10 +1265,11 @@ bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::ve
     const bool multi = scan && roots.size() >= 2;
     double ms_root = 0.0;
     if (scan) BCD_TRY(scan_roots(g, roots, qcol, &ms_root));
-    auto launch = [&](bool scan_mode, int64_t first, int64_t count) -> bc_status {
+    auto launch = [&](bool scan_mode, int64_t first, int64_t count, bool trial = false) -> bc_status {
         TravParams p;
         memset(&p, 0, sizeof(p));
         p.mode = scan_mode ? kModeScan : kModeSpd;
+        p.flags = trial ? kFlagTrial : 0;
         if (scan_mode) {
             p.rlev = ws.rlev;
             p.rdist = ws.rdist;
@@ -1298,16 +1303,20 @@ bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::ve
         unsigned long long ed = 0;
         BCD_TRY(src_kernel_applies(g, p) ? run_src_traversal(g, W, p, nullptr, &ed)
                                           : run_traversal(g, W, p, nullptr, &ed));
-        if (edges) *edges += ed;
+        if (edges && !g->last.scan_skipped) *edges += ed;
         return BC_OK;
     };
     if (edges) *edges = 0;
     std::vector<uint32_t> cal_flags(64, 0);
-    if (multi && g->accumulation == 4 && ntiles > 1) {
-        BCD_TRY(launch(true, 0, 1));
-        BCD_CUDA(cudaMemcpyAsync(cal_flags.data(), ws.qflags, 64 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        BCD_CUDA(cudaStreamSynchronize(s));
-        BCD_TRY(launch(g->last.vpairs * kScanPairCost <= g->last.tight, 1, ntiles - 1));
+    if (multi && g->accumulation == 4 && (ntiles > 1 || !g->weighted)) {
+        BCD_TRY(launch(true, 0, 1, !g->weighted));
+        if (g->last.scan_skipped) {
+            BCD_TRY(launch(false, 0, ntiles));
+        } else {
+            BCD_CUDA(cudaMemcpyAsync(cal_flags.data(), ws.qflags, 64 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+            BCD_CUDA(cudaStreamSynchronize(s));
+            if (ntiles > 1) BCD_TRY(launch(g->last.vpairs * kScanPairCost <= g->last.tight, 1, ntiles - 1));
+        }
     } else {
         BCD_TRY(launch(scan, 0, ntiles));
     }

@@ -494,8 +494,8 @@ __device__ __noinline__ void push_masks(int L, long long ccnt, long long gwarp, 
             };
             fetch(base);
             do {
-                int wv[U], j[U];
-                uint64_t nm[U][W];
+                int wv[U], j[U], etag[U];
+                uint64_t nm[U][W], early[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     wv[u] = wn[u];
@@ -503,8 +503,12 @@ __device__ __noinline__ void push_masks(int L, long long ccnt, long long gwarp, 
                     if (wv[u] >= 0) {
                         load_mask<W>(p.vs + (size_t)wv[u] * p.vs_stride, nm[u]);
                         if (MODE == kModeReach) {
+                            // one word per mask: the row is one sector, and the tag
+                            // joins this round of loads
                             uint64_t c[W];
                             load_mask<W>(p.vs + (size_t)wv[u] * p.vs_stride + cur * W, c);
+                            early[u] = p.vs[(size_t)wv[u] * p.vs_stride + nxt * W];
+                            etag[u] = p.tag[wv[u]];
 #pragma unroll
                             for (int w = 0; w < W; ++w) nm[u][w] |= c[w];
                         }
@@ -525,9 +529,15 @@ __device__ __noinline__ void push_masks(int L, long long ccnt, long long gwarp, 
                     int old = 0x7fffffff;
                     if (any) {
                         uint64_t *wrow = p.vs + (size_t)wv[u] * p.vs_stride + nxt * W;
-                        const int tg = p.tag[wv[u]];
                         uint64_t nx[W];
-                        load_mask<W>(wrow, nx);
+                        int tg;
+                        if (MODE == kModeReach) {
+                            nx[0] = early[u];
+                            tg = etag[u];
+                        } else {
+                            tg = p.tag[wv[u]];
+                            load_mask<W>(wrow, nx);
+                        }
                         bool add = false;
 #pragma unroll
                         for (int w = 0; w < W; ++w) {
@@ -683,6 +693,30 @@ __device__ __noinline__ void gather_level(int L, long long ics, long long iccnt,
     buf.st[lane].tight += tight;
     if (over) set_err(p.ctr, kDevWide);
 }
+
+// 1 / sigma. The chip's fp64 units are few (a warp instruction holds an SM's
+// for 16 cycles, so the dozen of a division cost more than the rest of a
+// step): counts up to kInverses, nearly all of them, are looked up.
+constexpr int kInverses = 2048;
+__device__ __forceinline__ double *inverses() {
+    __shared__ double s_inv[kInverses];
+    return s_inv;
+}
+__device__ __forceinline__ double inverse_of(const double *s_inv, uint32_t x) {
+    return x < (uint32_t)kInverses ? s_inv[x] : 1.0 / (double)x;
+}
+__device__ __forceinline__ double inverse_of(const double *s_inv, double x) { return 1.0 / x; }
+
+// a / sigma, the same bits as the fp64 division: with y the correctly rounded
+// 1 / sigma, q = a y and r = a - q sigma exactly, q + r y rounds to a / sigma
+// (Markstein, IBM J. Res. Dev. 34, 1990), four fp64 operations instead of a
+// division's dozen.
+__device__ __forceinline__ double quotient(const double *s_inv, double a, uint32_t x) {
+    if (x >= (uint32_t)kInverses) return a / (double)x;
+    const double y = s_inv[x], q = a * y;
+    return fma(fma(-q, (double)x, a), y, q);
+}
+__device__ __forceinline__ double quotient(const double *s_inv, double a, double x) { return a / x; }
 
 // Bookkeeping of the level-L entries after a bottom-up step (which counts
 // paths itself), one thread each.
@@ -840,15 +874,6 @@ __device__ __noinline__ void pull_level(int L, const uint64_t *s_valid, long lon
     if (over) set_err(p.ctr, kDevWide);
 }
 
-// 1 / sigma. The chip's fp64 units are few (a warp instruction holds an SM's
-// for 16 cycles, so the dozen of a division cost more than the rest of a
-// step): counts up to kInverses, nearly all of them, are looked up.
-constexpr int kInverses = 2048;
-__device__ __forceinline__ double inverse_of(const double *s_inv, uint32_t x) {
-    return x < (uint32_t)kInverses ? s_inv[x] : 1.0 / (double)x;
-}
-__device__ __forceinline__ double inverse_of(const double *s_inv, double x) { return 1.0 / x; }
-
 // Eq. 4, push form, from level L into level L - 1: each entry w of level L
 // sends c_s(w) = (1 + delta_s(w)) / sigma_s(w) = 1 / sigma_s(w) + acc_s(w)
 // (delta_s(w) = sigma_s(w) * acc_s(w), complete: level L + 1 pushed into it in
@@ -1002,6 +1027,7 @@ __device__ void level_outputs(const TravParams &p, int L, bool swap, bool set_ne
 template <int W, typename T>
 __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_need, long long gwarp,
                             long long nwarps) {
+    const double *const s_inv = inverses();
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
     const int lane = threadIdx.x & 31;
@@ -1066,11 +1092,11 @@ __device__ void vertex_scan(const TravParams &p, int Lmax, const uint64_t *s_nee
                     for (int ii = 0; ii < PL; ++ii) {
                         const int s = lane + 32 * ii;
                         if (ks[ii] == k0 && mask_bit<W>(f0, s)) {
-                            a[ii] += r0 / (double)q0[s];
+                            a[ii] += quotient(s_inv, r0, q0[s]);
                             ++pairs;
                         }
                         if (ks[ii] == k1 && mask_bit<W>(f1, s)) {
-                            a[ii] += r1 / (double)q1[s];
+                            a[ii] += quotient(s_inv, r1, q1[s]);
                             ++pairs;
                         }
                     }
@@ -1096,6 +1122,61 @@ struct ScanBuf {
     int32_t ql[64 * W * G];                   // d(s, r_c) for sources that need column c, else -1
 };
 
+// The number of terms vertex_scan_multi would add up, without adding them: an
+// entry (t, F) of level L has, for column c, the sources of F that meet r_c at
+// level L - d(r_c, t). lm holds these sources per (column, level), the levels
+// from 63 on in one place (an upper bound there). One thread per entry.
+template <int W>
+struct CountBuf {
+    static constexpr int G = ScanBuf<W>::G;
+    unsigned long long lm[G][64][W];
+};
+template <int W>
+__device__ __noinline__ void scan_count(int Lmax, long long gthr, long long nthr) {
+    constexpr int S = 64 * W;
+    constexpr int G = CountBuf<W>::G;
+    const TravParams &p = shared_params();
+    const uint64_t *s_need = tile_need();
+    CountBuf<W> &cb = *reinterpret_cast<CountBuf<W> *>(s_dyn + kParamBytes + 512 * W);
+    unsigned long long pairs = 0;
+    for (int cg = 0; cg < p.ncols; cg += G) {
+        const int nc = min(G, p.ncols - cg);
+        __syncthreads();
+        for (int i = threadIdx.x; i < G * 64 * W; i += blockDim.x) (&cb.lm[0][0][0])[i] = 0ull;
+        __syncthreads();
+        for (int s = threadIdx.x; s < S; s += blockDim.x) {
+            uint64_t x = s_need[s];
+            while (x) {
+                const int q = __ffsll((long long)x) - 1;
+                x &= x - 1;
+                const int j = p.qcol[q] - cg;
+                if (j < 0 || j >= nc) continue;
+                const int lv = p.qlevel[s * 64 + q];
+                if (lv >= 1) atomicOr(&cb.lm[j][min(lv, 63)][s >> 6], 1ull << (s & 63));
+            }
+        }
+        __syncthreads();
+        for (int L = 2; L <= Lmax; ++L) {
+            const long long eend = p.lev_start[L + 1];
+            for (long long e = p.lev_start[L] + gthr; e < eend; e += nthr) {
+                const int32_t *row = p.rlevq + (size_t)p.hv[e] * 64 + cg;
+                uint64_t F[W];
+                load_mask<W>(p.hm + (size_t)e * W, F);
+                for (int j = 0; j < nc; ++j) {
+                    const int dr = row[j];
+                    if (dr < 1 || dr >= L) continue;
+                    const unsigned long long *m = cb.lm[j][min(L - dr, 63)];
+#pragma unroll
+                    for (int w = 0; w < W; ++w) pairs += (unsigned)__popcll(F[w] & m[w]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(kFull, pairs, o);
+    if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&p.ctr->trial_pairs, pairs);
+}
+
 // Dependencies on several query vertices at once by the vertex scan: the
 // form of vertex_scan for a group whose queries sit at up to 64 distinct
 // vertices (columns c, vertex croot[c]). rlevq / rsigq [t * 64 + c] hold
@@ -1114,6 +1195,7 @@ __device__ __noinline__ void vertex_scan_multi(int Lmax, long long gwarp, long l
     const TravParams &p = shared_params();
     const uint64_t *s_need = tile_need();
     ScanBuf<W> &sb = *reinterpret_cast<ScanBuf<W> *>(s_dyn + kParamBytes + 512 * W);
+    const double *const s_inv = inverses();
     constexpr int S = 64 * W;
     constexpr int PL = 2 * W;
     constexpr int G = ScanBuf<W>::G;
@@ -1163,9 +1245,12 @@ __device__ __noinline__ void vertex_scan_multi(int Lmax, long long gwarp, long l
             if (kmax[j] >= 1) lfrom = min(lfrom, kmin[j] + 1);
         }
         for (int L = lfrom; L <= Lmax; ++L) {
-            const long long eend = p.lev_start[L + 1];
-            for (long long b = p.lev_start[L] + 32 * gwarp; b < eend; b += 32 * nwarps) {
-                const long long e = b + lane;
+            const long long ebeg = p.lev_start[L], eend = p.lev_start[L + 1];
+            // entries a warp takes together: fewer on thin levels, where a warp's
+            // kept (entry, column) pairs, one after another, are what it waits for
+            const int wide = (int)min(32ll, (eend - ebeg + nwarps - 1) / nwarps);
+            for (long long b = ebeg + wide * gwarp; b < eend; b += wide * nwarps) {
+                const long long e = lane < wide ? b + lane : eend;
                 int t = 0;
                 unsigned kq = 0;
                 int dr[G];
@@ -1215,7 +1300,7 @@ __device__ __noinline__ void vertex_scan_multi(int Lmax, long long gwarp, long l
                         for (int ii = 0; ii < PL; ++ii) {
                             const int s = lane + 32 * ii;
                             if (mask_bit<W>(F, s) && s_ql[s * G + j] == k) {
-                                atomicAdd(&s_acc[s * G + j], rs / (double)qs[s]);
+                                atomicAdd(&s_acc[s * G + j], quotient(s_inv, rs, qs[s]));
                                 ++pairs;
                             }
                         }
@@ -1302,8 +1387,8 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
     __shared__ uint64_t s_active_next[W];
     __shared__ uint64_t s_valid[W];  // the tile's occupied source slots
     __shared__ int32_t s_lstop;
-    __shared__ double s_inv[MODE == kModeSpd ? kInverses : 1];  // Eq. 4: 1 / k
-    if (MODE == kModeSpd)
+    double *const s_inv = inverses();  // 1 / k
+    if (MODE != kModeReach && sizeof(T) == 4)
         for (int i = threadIdx.x; i < kInverses; i += blockDim.x) s_inv[i] = 1.0 / (double)max(i, 1);
     const bool timer = team == 0 && leader;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
@@ -1410,6 +1495,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
         }
         if (leader) atomicMax(&p.ctr->levels_max, (unsigned long long)Lmax);
 
+        bool skipped = false;  // a scan on trial that was not made
         // the scan over several query vertices takes the warps' buffers
         if (MODE == kModeScan) flush_stats(p.ctr, warp_buf<W>().st[lane], lane);
 
@@ -1437,7 +1523,19 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             }
             if (!team_barrier(p, gen)) return;
         } else if (MODE == kModeScan && !(p.flags & kFlagNoBackward)) {
-            if (p.ncols >= 2)
+            if (p.flags & kFlagTrial) {
+                // a lone tile on trial: its terms are counted first, and when they
+                // are too many the tile is left to the Eq. 4 pass
+                scan_count<W>(Lmax, gthr, nthr);
+                if (!team_barrier(p, gen)) return;
+                if (scan_too_long(ld_vol(&p.ctr->trial_pairs), ld_vol(&p.ctr->tight))) {
+                    if (leader) p.ctr->scan_skipped = 1ull;
+                    skipped = true;
+                }
+            }
+            if (skipped)
+                ;
+            else if (p.ncols >= 2)
                 vertex_scan_multi<W, T>(Lmax, gwarp, nwarps);
             else
                 vertex_scan<W, T>(p, Lmax, s_need, gwarp, nwarps);
@@ -1511,7 +1609,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
         if (MODE == kModeSpd) flush_stats(p.ctr, warp_buf<W>().st[lane], lane);
 
         // ---------------- tile end ----------------
-        if (MODE == kModeScan && block == 0) {
+        if (MODE == kModeScan && block == 0 && !skipped) {
             // one sum per source (one query vertex) or per (source, column)
             for (int s = threadIdx.x; s < S; s += blockDim.x) {
                 uint64_t x = s_need[s];
@@ -1524,7 +1622,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             }
             __syncthreads();
         }
-        if (MODE != kModeReach && block == 0) tile_query_sums(p, tile, S, tsrc, s_need);
+        if (MODE != kModeReach && block == 0 && !skipped) tile_query_sums(p, tile, S, tsrc, s_need);
         if (MODE == kModeReach) {
             for (long long e = gthr; e < total; e += nthr)
                 atomicOr((unsigned long long *)&p.rvmask[p.hv[e]], (unsigned long long)p.hm[e * W]);
@@ -1601,17 +1699,19 @@ bc_status launch(bc_graph *g, TravParams &p) {
     const int threads = g->block_threads;
     if (threads < 64 * W) return set_error(BC_E_INVALID_ARG, "block_threads must be at least 64 * tile_words");
     size_t smem = sizeof(WarpBuf<W>) * (size_t)(threads / 32);
-    if (MODE == kModeScan) smem = std::max(smem, sizeof(ScanBuf<W>));
+    if (MODE == kModeScan) smem = std::max(smem, std::max(sizeof(ScanBuf<W>), sizeof(CountBuf<W>)));
     smem += kParamBytes + 512 * W;
     int per_sm = 0;
     BCD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) return set_error(BC_E_INTERNAL, "traversal kernel cannot be resident");
-    const int blocks = g->num_sms * per_sm;
+    // reach traversals of small graphs: blocks without work would only lengthen
+    // the barriers
+    int blocks = g->num_sms * per_sm;
+    if (MODE == kModeReach) blocks = (int)std::max<int64_t>(std::min<int64_t>(blocks, 16), std::min<int64_t>(blocks, g->m / 2048));
     p.nteams = (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min(g->ws.teams, blocks), p.ntiles));
     p.team_blocks = blocks / p.nteams;
     dim3 grid((unsigned)(p.nteams * p.team_blocks)), block((unsigned)threads);
-    BCD_CUDA(cudaMemsetAsync(p.bar, 0, sizeof(TeamBar) * (size_t)p.nteams, g->stream));
     void *args[] = {(void *)&p};
     BCD_CUDA(cudaLaunchCooperativeKernel((const void *)kern, grid, block, args, smem, g->stream));
     g->launches += 1;
@@ -1717,7 +1817,7 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         p.hcap = p.mode == kModeReach ? ws.hmcap : ws.hcap;
         p.hm_words = ws.hcap * ws.W;
         p.ws_slots = 64 * ws.W;
-        p.bar = ws.bar;
+        p.bar = reinterpret_cast<TeamBar *>(reinterpret_cast<char *>(ws.ctr) + kCounterBytes);
         p.nteams = 1;
         p.team_blocks = 1;
         p.chunks = ws.chunks;
@@ -1745,7 +1845,8 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
             p.npchunks = ws.npchunks;
             p.pull_arcs_min = std::max<int64_t>(1, (int64_t)((double)g->m * g->pull_permille / 1000.0));
         }
-        BCD_CUDA(cudaMemsetAsync(ws.ctr, 0, sizeof(Counters), g->stream));
+        // the counters and, behind them, the teams' barrier words
+        BCD_CUDA(cudaMemsetAsync(ws.ctr, 0, kCounterBytes + sizeof(TeamBar) * (size_t)ws.teams, g->stream));
         bc_status st = BC_E_INTERNAL;
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         const bool timed = cudaEventCreate(&ev0) == cudaSuccess && cudaEventCreate(&ev1) == cudaSuccess;
