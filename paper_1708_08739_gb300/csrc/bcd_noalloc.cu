@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "bcd.h"
@@ -19,12 +20,23 @@ namespace {
 
 constexpr int32_t kMaxN = BC_NOALLOC_MAX_VERTICES;
 constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kArcs = 4;         // arcs a lane has in flight
+constexpr int kLongRow = 1024;   // longer rows are walked by a whole block
+
+// Frontier of one level: its short rows are queued from the front of the
+// level's buffer and its long ones from the back (a vertex is queued once, so
+// they never meet), each drawn from a counter.
+struct Frontier {
+    uint32_t shorts, longs;        // queued
+    uint32_t next_short, next_long;  // handed out past the first of each warp / block
+};
 
 struct NoallocScratch {
     uint32_t visited[kMaxN / 32];   // one bit per vertex
     int32_t queue[2][kMaxN];        // frontier of the current / next level
     int64_t block_count[1024];      // per-block counts for the ordered output
-    uint32_t qlen[2];               // frontier sizes
+    Frontier front[3];              // of the current, the next and the level after (being cleared)
     uint32_t bar_count;
     uint32_t bar_gen;
     int32_t err;
@@ -76,97 +88,195 @@ __device__ bool grid_sync(NoallocScratch *s, uint32_t &gen) {
     return ok;
 }
 
-__global__ void __launch_bounds__(kThreads) rv_noalloc_kernel(NoallocScratch *s, const int64_t *roff,
-                                                               const int32_t *rcol, int32_t n, int32_t r,
-                                                               int32_t *out, int64_t cap) {
+// Marks the heads y (negative: none) and queues the ones not seen before, short
+// rows and long rows apart, with one counter atomic per warp and kind.
+__device__ __forceinline__ void visit(NoallocScratch *s, const int64_t *roff, int next, Frontier *f,
+                                      const int32_t (&y)[kArcs], int lane) {
+    uint32_t word[kArcs];
+#pragma unroll
+    for (int k = 0; k < kArcs; ++k) word[k] = y[k] >= 0 ? __ldcg(&s->visited[y[k] >> 5]) : ~0u;
+#pragma unroll
+    for (int k = 0; k < kArcs; ++k) {
+        bool fresh = false, lng = false;
+        const uint32_t bit = 1u << (y[k] & 31);
+        if (!(word[k] & bit)) fresh = !(atomicOr(&s->visited[y[k] >> 5], bit) & bit);
+        if (!__any_sync(0xffffffffu, fresh)) continue;
+        if (fresh) lng = roff[y[k] + 1] - roff[y[k]] > kLongRow;
+        const unsigned ms = __ballot_sync(0xffffffffu, fresh && !lng), ml = __ballot_sync(0xffffffffu, lng);
+        uint32_t bs = 0, bl = 0;
+        if (lane == 0) {
+            if (ms) bs = atomicAdd(&f->shorts, (uint32_t)__popc(ms));
+            if (ml) bl = atomicAdd(&f->longs, (uint32_t)__popc(ml));
+        }
+        bs = __shfl_sync(0xffffffffu, bs, 0);
+        bl = __shfl_sync(0xffffffffu, bl, 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (lng)
+            s->queue[next][kMaxN - 1 - (bl + __popc(ml & below))] = y[k];
+        else if (fresh)
+            s->queue[next][bs + __popc(ms & below)] = y[k];
+    }
+}
+
+// Level-synchronous BFS over R(G), one grid barrier per level. A warp draws up
+// to 32 frontier vertices and packs their arcs onto its lanes, kArcs per lane in
+// flight; rows of more than kLongRow arcs go to whole blocks. On R-MAT 22 with
+// reciprocal arcs one warp per vertex, with one counter atomic per discovered
+// vertex, took 5.2 ms: its longest rows, tens of thousands of arcs behind one
+// warp, were the time of a level.
+__global__ void __launch_bounds__(kThreads, 2) rv_noalloc_kernel(NoallocScratch *s, const int64_t *roff,
+                                                                  const int32_t *rcol, int32_t n, int32_t r,
+                                                                  int32_t *out, int64_t cap) {
+    __shared__ int s_incl[kWarps][32];
+    __shared__ long long s_off[kWarps][32];
+    __shared__ uint32_t s_long;
     uint32_t gen = 0;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nthr = (long long)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t gw = blockIdx.x * kWarps + warp, nw = gridDim.x * kWarps;
     const int words = (n + 31) / 32;
-    for (long long i = tid; i < words; i += nthr) s->visited[i] = 0u;
+    int *incl = s_incl[warp];
+    long long *off = s_off[warp];
+    for (long long i = tid; i < words; i += nthr) s->visited[i] = i == (r >> 5) ? 1u << (r & 31) : 0u;
     if (tid == 0) {
-        s->qlen[0] = 1;
-        s->qlen[1] = 0;
-        s->queue[0][0] = r;
+        const bool lng = roff[r + 1] - roff[r] > kLongRow;
+        s->queue[0][lng ? kMaxN - 1 : 0] = r;
+        s->front[0].shorts = lng ? 0u : 1u;
+        s->front[0].longs = lng ? 1u : 0u;
     }
     if (!grid_sync(s, gen)) return;
-    if (tid == 0) atomicOr(&s->visited[r >> 5], 1u << (r & 31));
-    if (!grid_sync(s, gen)) return;
-    int cur = 0;
-    // level-synchronous BFS over R(G); one warp per frontier vertex
-    for (;;) {
-        const uint32_t len = *(volatile uint32_t *)&s->qlen[cur];
-        const long long gw = tid >> 5, nw = nthr >> 5;
-        for (long long i = gw; i < len; i += nw) {
-            const int32_t x = __ldcg(&s->queue[cur][i]);
+    for (int level = 0;; ++level) {
+        Frontier *cf = &s->front[level % 3], *nf = &s->front[(level + 1) % 3];
+        const int cur = level & 1;
+        const uint32_t shorts = __ldcg(&cf->shorts), longs = __ldcg(&cf->longs);
+        if (shorts + longs == 0u) break;
+        if (tid == 0) s->front[(level + 2) % 3] = Frontier{0u, 0u, 0u, 0u};
+        // long rows: a block each, its first fixed, the others drawn
+        for (uint32_t i = blockIdx.x; i < longs;) {
+            const int32_t x = __ldcg(&s->queue[cur][kMaxN - 1 - i]);
             const long long b = roff[x], e = roff[x + 1];
-            for (long long a = b + lane; a < e; a += 32) {
-                const int32_t y = rcol[a];
-                const uint32_t bit = 1u << (y & 31);
-                if (!(s->visited[y >> 5] & bit)) {
-                    const uint32_t old = atomicOr(&s->visited[y >> 5], bit);
-                    if (!(old & bit)) {
-                        const uint32_t pos = atomicAdd(&s->qlen[cur ^ 1], 1u);
-                        s->queue[cur ^ 1][pos] = y;
-                    }
+            for (long long a0 = b; a0 < e; a0 += kThreads * kArcs) {
+                int32_t y[kArcs];
+#pragma unroll
+                for (int k = 0; k < kArcs; ++k) {
+                    const long long a = a0 + k * kThreads + threadIdx.x;
+                    y[k] = a < e ? __ldcs(rcol + a) : -1;
                 }
+                visit(s, roff, cur ^ 1, nf, y, lane);
             }
+            __syncthreads();
+            if (threadIdx.x == 0) s_long = gridDim.x + atomicAdd(&cf->next_long, 1u);
+            __syncthreads();
+            i = s_long;
+        }
+        // short rows: groups of vertices, a warp's first fixed, the others drawn
+        const uint32_t group = max(1u, min(32u, shorts / (nw * 4u)));
+        for (uint32_t g0 = gw * group; g0 < shorts;) {
+            long long b = 0;
+            int len = 0;
+            if (lane < group && g0 + lane < shorts) {
+                const int32_t x = __ldcg(&s->queue[cur][g0 + lane]);
+                b = roff[x];
+                len = (int)(roff[x + 1] - b);
+            }
+            int in = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int z = __shfl_up_sync(0xffffffffu, in, o);
+                if (lane >= o) in += z;
+            }
+            incl[lane] = in;
+            off[lane] = b - (in - len);
+            const int total = __shfl_sync(0xffffffffu, in, 31);
+            __syncwarp();
+            for (int base = 0; base < total; base += 32 * kArcs) {
+                int32_t y[kArcs];
+#pragma unroll
+                for (int k = 0; k < kArcs; ++k) {
+                    const int i = base + 32 * k + lane;
+                    int v = 0;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (incl[v + o - 1] <= i) v += o;
+                    y[k] = i < total ? __ldcs(rcol + off[v] + i) : -1;
+                }
+                visit(s, roff, cur ^ 1, nf, y, lane);
+            }
+            __syncwarp();
+            const uint32_t drawn = nw * group;
+            uint32_t g = shorts;
+            if (drawn < shorts) {
+                if (lane == 0) g = drawn + atomicAdd(&cf->next_short, group);
+                g = __shfl_sync(0xffffffffu, g, 0);
+            }
+            g0 = g;
         }
         if (!grid_sync(s, gen)) return;
-        const uint32_t next = *(volatile uint32_t *)&s->qlen[cur ^ 1];
-        if (next == 0) break;
-        if (tid == 0) s->qlen[cur] = 0;
-        if (!grid_sync(s, gen)) return;
-        cur ^= 1;
     }
-    // ordered output: per-block bit counts, one-block scan, per-block writes
-    const long long per = (words + gridDim.x - 1) / gridDim.x;
-    const long long w0 = (long long)blockIdx.x * per, w1 = min((long long)words, w0 + per);
-    __shared__ long long s_cnt;
-    if (threadIdx.x == 0) s_cnt = 0;
-    __syncthreads();
-    for (long long w = w0 + threadIdx.x; w < w1; w += blockDim.x) {
+    // ordered output: counts per warp and block, every block sums the blocks
+    // before it, every warp writes its words
+    const int per = (words + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int wper = (per + kWarps - 1) / kWarps;
+    const int w0 = min(words, (int)blockIdx.x * per + warp * wper);
+    const int w1 = min(min(words, ((int)blockIdx.x + 1) * per), w0 + wper);
+    __shared__ int s_cnt[kWarps];
+    __shared__ long long s_base;
+    int mine = 0;
+    for (int w = w0 + lane; w < w1; w += 32) {
         uint32_t x = __ldcg(&s->visited[w]);
         if (w == (r >> 5)) x &= ~(1u << (r & 31));
-        atomicAdd((unsigned long long *)&s_cnt, (unsigned long long)__popc(x));
+        mine += __popc(x);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if (lane == 0) s_cnt[warp] = mine;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long c = 0;
+        for (int w = 0; w < kWarps; ++w) c += s_cnt[w];
+        s->block_count[blockIdx.x] = c;
+    }
+    if (!grid_sync(s, gen)) return;
+    if (warp == 0) {
+        long long before = 0, all = 0;
+        for (int k = lane; k < (int)gridDim.x; k += 32) {
+            const long long c = __ldcg(&s->block_count[k]);
+            all += c;
+            if (k < (int)blockIdx.x) before += c;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        if (lane == 0) {
+            s_base = all > cap ? -1 : before;
+            if (blockIdx.x == 0) s->total = all;
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 0) s->block_count[blockIdx.x] = s_cnt;
-    if (!grid_sync(s, gen)) return;
-    if (tid == 0) {
-        long long run = 0;
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            const long long c = __ldcg(&s->block_count[b]);
-            s->block_count[b] = run;
-            run += c;
+    if (s_base < 0) return;
+    long long base = s_base;
+    for (int w = 0; w < warp; ++w) base += s_cnt[w];
+    for (int v0 = w0; v0 < w1; v0 += 32) {
+        const int w = v0 + lane;
+        uint32_t x = w < w1 ? __ldcg(&s->visited[w]) : 0u;
+        if (w == (r >> 5)) x &= ~(1u << (r & 31));
+        const int c = __popc(x);
+        int in = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int z = __shfl_up_sync(0xffffffffu, in, o);
+            if (lane >= o) in += z;
         }
-        s->total = run;
-    }
-    if (!grid_sync(s, gen)) return;
-    const long long total = *(volatile long long *)&s->total;
-    if (total > cap) return;
-    // each block writes its words in order; one warp walks the block's range
-    if (threadIdx.x < 32) {
-        long long base = __ldcg(&s->block_count[blockIdx.x]);
-        for (long long w0b = w0; w0b < w1; w0b += 32) {
-            const long long w = w0b + lane;
-            uint32_t x = w < w1 ? __ldcg(&s->visited[w]) : 0u;
-            if (w == (r >> 5)) x &= ~(1u << (r & 31));
-            const int c = __popc(x);
-            int incl = c;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            long long pos = base + incl - c;
-            while (x) {
-                const int b = __ffs(x) - 1;
-                x &= x - 1;
-                out[pos++] = (int32_t)(w * 32 + b);
-            }
-            base += __shfl_sync(0xffffffffu, incl, 31);
+        long long pos = base + in - c;
+        while (x) {
+            const int b = __ffs(x) - 1;
+            x &= x - 1;
+            out[pos++] = w * 32 + b;
         }
+        base += __shfl_sync(0xffffffffu, in, 31);
     }
 }
 
@@ -201,14 +311,15 @@ extern "C" bc_status bc_rv_compute_noalloc(const int64_t *d_roffsets, const int3
             BCD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             BCD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rv_noalloc_kernel, kThreads, 0));
             if (per_sm < 1) return bcd::set_error(BC_E_INTERNAL, "bc_rv_compute_noalloc: kernel cannot be resident");
-            g_grid[dev] = sms < 1024 ? sms : 1024;
+            g_grid[dev] = std::min(sms * std::min(per_sm, 2), 1024);
             g_addr[dev] = (NoallocScratch *)p;
         }
         s = g_addr[dev];
-        grid = g_grid[dev];
+        // blocks without work would only lengthen the barriers
+        grid = std::min(g_grid[dev], std::max(8, n / 2048));
     }
     cudaStream_t st = (cudaStream_t)stream;
-    BCD_CUDA(cudaMemsetAsync(&s->qlen, 0, sizeof(uint32_t) * 4 + sizeof(int32_t) * 2, st));
+    BCD_CUDA(cudaMemsetAsync(&s->front[0], 0, sizeof(Frontier) * 3 + sizeof(uint32_t) * 2 + sizeof(int32_t) * 2, st));
     void *args[] = {(void *)&s, (void *)&d_roffsets, (void *)&d_rcols, (void *)&n, (void *)&r, (void *)&d_out,
                     (void *)&cap};
     BCD_CUDA(cudaLaunchCooperativeKernel((const void *)rv_noalloc_kernel, dim3(grid), dim3(kThreads), args, 0, st));

@@ -1,0 +1,38 @@
+"""The allocation-free RV(r) kernel at the sizes where its split changes:
+vertex counts around whole words and warps, rows around the length from which
+a block walks them, long chains (many levels), and an empty reach set. Lists
+bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+import oracle as O
+from helpers import csr
+
+pytestmark = pytest.mark.gpu
+
+
+def fan(n, row):
+    """A chain 0 <- 1 <- 2 ... and a vertex with `row` in-arcs (from the last
+    vertices) in its middle."""
+    arcs = {(i + 1, i) for i in range(min(n - 1, 40))}
+    hub = min(n - 1, 20)
+    arcs |= {(n - 1 - i, hub) for i in range(min(row, n - 1)) if n - 1 - i != hub}
+    return sorted(arcs)
+
+
+@pytest.mark.parametrize("n,row", [(1, 0), (2, 0), (31, 3), (32, 3), (33, 3), (1100, 1023), (1100, 1024), (1100, 1025),
+                                   (5000, 2049), (40000, 30000), (100001, 60000)])
+def test_noalloc_edges(n, row):
+    torch = pytest.importorskip("torch")
+    import paper_1708_08739_gb300 as bcd
+    g = csr(n, fan(n, row) if n > 1 else [])
+    og = O.Graph.from_csr(g)
+    roff, rcol = torch.from_numpy(og.roff.copy()).cuda(), torch.from_numpy(og.rcol.copy()).cuda()
+    if rcol.numel() == 0:
+        rcol = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.full((n + 1,), -7, dtype=torch.int32, device="cuda")
+    for r in sorted({0, n - 1, n // 2, min(n - 1, 20)}):
+        want = O.rv(og, r)
+        k = bcd.bc_rv_compute_noalloc(roff.data_ptr(), rcol.data_ptr(), n, r, out.data_ptr(), n,
+                                      torch.cuda.current_stream().cuda_stream)
+        assert k == want.shape[0] and np.array_equal(out[:k].cpu().numpy(), want), (n, row, r)
