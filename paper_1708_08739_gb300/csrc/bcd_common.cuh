@@ -275,6 +275,11 @@ struct bcd_workspace {
     uint32_t *qflags = nullptr;   // [64]
     uint64_t *srcflag = nullptr;  // [W]
     // weighted source kernel (one source per block): per-block state
+    int32_t *spos = nullptr;               // [n] position of a vertex in the state (by in-degree)
+    int32_t *sinv = nullptr;               // [n] vertex at a position
+    int64_t *srow = nullptr;               // [2 n] bounds of its row
+    int32_t *scol = nullptr;               // [m] heads as positions
+    int32_t sheads = 0;                    // positions of vertices with in-arcs (the first ones)
     int32_t sblocks = 0;                   // blocks the state is sized for
     unsigned long long *sds = nullptr;     // [sblocks * n * 2]: (distance, sigma) of each vertex
     uint32_t *stb = nullptr;               // [sblocks * (m + 31) / 32]: tight-candidate arc bits

@@ -19,6 +19,13 @@
 // each, with their queued / consumed counters in shared memory. Eq. 4
 // launches also keep one bit per arc (see src_relax).
 //
+// The state is indexed by position, not by vertex: positions sort the vertices
+// by their in-degree's power of two, largest first (src_order). A relaxation
+// touches a vertex once per in-arc, so the sectors that are touched most hold
+// nothing else, and the vertices that no arc leads to (half of an R-MAT graph)
+// take no room among the others. The heads of the arcs are kept as positions in
+// a copy of the column array, the rows' bounds in one 16-byte pair per position.
+//
 // Sigma rides along the relaxations. Settling u at distance d (its sigma is
 // final: every predecessor on a shortest path sits at a smaller distance and
 // relaxed its arcs in an earlier level), each out-arc (u, v, w) offers the
@@ -29,8 +36,8 @@
 // pair holds its distance with the sum over exactly its tight in-arcs (sigma
 // values are integers: exact in any order below 2^53). Every arc is read
 // once in the forward pass, along its tail's out-row; no in-arc pass.
-// Where it fits, shared memory holds one bit per vertex: settled for the
-// current source. An arc to a settled vertex can change nothing, and most arcs
+// Where it fits, shared memory holds one bit per vertex that arcs lead to (the
+// first positions): settled for the current source. An arc to a settled vertex can change nothing, and most arcs
 // are such (they lead to hubs, which settle early), so their heads' distances,
 // random 32-byte sectors each, are not read.
 // A vertex queued in the slot of d whose distance has since dropped is stale
@@ -75,8 +82,10 @@ constexpr int kPackRows = 4;
 // Threads of the largest block (one per SM at 64 registers); see src_threads.
 constexpr int kSrcThreads = 1024;
 // Dynamic shared memory of a block (227 KB less the static arrays): the warps'
-// staging, the ring's counters and, up to about 1.6 million vertices, the
-// settled bits.
+// staging, the ring's counters and, up to about 1.6 million vertices with
+// in-arcs, the settled bits. (16-bit distance bounds of the first positions in
+// what is left, to skip more reads, took the L1 cache that the register spills
+// need: R-MAT 20 277 -> 420 ms at 224 KB, 264-272 ms at 32 to 64 KB.)
 constexpr size_t kSrcDynSmem = 224 * 1024;
 constexpr double kSrcTwo53 = 9007199254740992.0;
 
@@ -99,6 +108,11 @@ struct SrcParams {
     double *sdep;               // [nsrc * 64]
     uint32_t *sflag;            // [nsrc] sigma >= 2^53 seen
     unsigned long long *next;   // source hand-out
+    const int32_t *col;         // [m] heads, as positions
+    const longlong2 *row;       // [n] arcs [x, y) of the vertex at a position
+    const int32_t *pos;         // [n] position of a vertex
+    const int32_t *inv;         // [n] vertex at a position
+    int32_t heads;              // positions of vertices with in-arcs
     int64_t n;
     int64_t bcap;               // power of two
     int64_t chcap;
@@ -259,7 +273,7 @@ template <class PairT, bool kBits>
 __device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, uint32_t *bk, uint32_t *s_cnt,
                                           const uint32_t *s_done, uint32_t *tb, int64_t bcap, int R,
                                           unsigned long long d, const WarpArcs &wa, int total,
-                                          unsigned long long &adds) {
+                                          const int32_t *col, unsigned long long &adds) {
     const int lane = threadIdx.x & 31;
     int err = 0;
     for (int base = lane; base < total; base += 32 * kLanesBatch) {
@@ -277,7 +291,7 @@ __device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, u
             y[j] = -1;
             if (i < total) {
                 const long long a = wa.off[v] + i;
-                y[j] = __ldg(p.col + a);
+                y[j] = __ldg(col + a);
                 w[j] = __ldg(p.wt + a);
             }
         }
@@ -323,7 +337,7 @@ __device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, u
 // Sum of c(y) over the tight out-arcs (y at distance d + w(v, y)) among arcs
 // [a, ae) of a vertex at distance d, this lane's share: the words rl, rl + lpp,
 // ... of the row's arc bits. Only arcs whose bit the forward set can be tight.
-__device__ __forceinline__ double src_pull_c(const TravParams &p, const DistSig *ds, const uint32_t *tb,
+__device__ __forceinline__ double src_pull_c(const TravParams &p, const int32_t *col, const DistSig *ds, const uint32_t *tb,
                                              unsigned long long d, long long a, long long ae, int rl, int lpp) {
     double acc = 0.0;
     if (ae <= a) return acc;
@@ -343,7 +357,7 @@ __device__ __forceinline__ double src_pull_c(const TravParams &p, const DistSig 
                 bits &= bits - 1u;
                 if (ok[j]) {
                     want[j] = d + __ldg(p.wt + aj);
-                    v[j] = ds[__ldg(p.col + aj)];
+                    v[j] = ds[__ldg(col + aj)];
                 }
             }
 #pragma unroll
@@ -380,11 +394,11 @@ __device__ __forceinline__ void src_store_chunks(Chunk *chs, long long c0, int v
 
 // delta(v) = sigma(v) * acc; c(v) = (1 + delta(v)) / sigma(v) = 1 / sigma(v) +
 // acc replaces sigma(v).
-__device__ __forceinline__ void src_finalize(const TravParams &p, DistSig *ds, uint64_t need, double *s_dep, int v,
-                                             double acc) {
+__device__ __forceinline__ void src_finalize(const TravParams &p, const int32_t *inv, DistSig *ds, uint64_t need, double *s_dep,
+                                             int v, double acc) {
     const double sv = ds[v].s;
     ds[v].s = 1.0 / sv + acc;
-    uint64_t y = __ldg(p.qmask + v) & need;
+    uint64_t y = __ldg(p.qmask + __ldg(inv + v)) & need;
     while (y) {
         const int q = __ffsll((long long)y) - 1;
         y &= y - 1;
@@ -417,8 +431,8 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
     uint32_t *s_ring = reinterpret_cast<uint32_t *>(s_src + sizeof(WarpArcs) * (blockDim.x >> 5));  // [2 * R]: queued, then consumed, per slot
     uint32_t *s_cnt = s_ring;
     uint32_t *s_base = s_ring + R;
-    uint32_t *s_done = s_ring + 2 * R;  // [(n + 31) / 32]
-    const int done_words = kBits ? (int)((q.n + 31) / 32) : 0;
+    uint32_t *s_done = s_ring + 2 * R;  // [(heads + 31) / 32]
+    const int done_words = kBits ? (q.heads + 31) / 32 : 0;
     const size_t boff = (size_t)blockIdx.x * (size_t)q.n;
     DistSig *ds = q.ds + boff;  // wide pairs (Eq. 4 reads and writes them directly)
     PairT P;
@@ -472,8 +486,9 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
         if (v0 < 0) continue;
         const uint64_t need = __ldg(p.need + v0);
         if (tid == 0) {
-            P.seed(v0);
-            bk[0] = (uint32_t)v0;  // slot 0, position 0
+            const int x0 = __ldg(q.pos + v0);
+            P.seed(x0);
+            bk[0] = (uint32_t)x0;  // slot 0, position 0
             s_cnt[0] = 1u;
         }
         __syncthreads();
@@ -534,10 +549,11 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     if (lane < gsize && (uint32_t)(g0 + lane) < cnt) {
                         x = (int)bks[(b0 + (uint32_t)(g0 + lane)) & (uint32_t)(bcap - 1)];
                         P.get(x, xd, xs);
-                        rb = __ldg(p.off + x);
-                        re = __ldg(p.off + x + 1);
+                        const longlong2 row = __ldg(q.row + x);
+                        rb = row.x;
+                        re = row.y;
                         seen = *(volatile const int32_t *)(p.tag + x);
-                        qm = __ldg(p.qmask + x);
+                        qm = __ldg(p.qmask + __ldg(q.inv + x));
                     }
                     const bool ok = xd == d;
                     const unsigned am = __ballot_sync(kFull, ok);
@@ -549,19 +565,13 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     if (ok) {
                         const long long deg = re - rb;
                         hv[eb + __popc(am & ((1u << lane) - 1u))] = x;
-                        if (kBits) atomicOr(&s_done[x >> 5], 1u << (x & 31));
+                        if (kBits && x < q.heads) atomicOr(&s_done[x >> 5], 1u << (x & 31));
                         st.reached += 1;
                         st.edges += (unsigned long long)deg;
                         if (PairT::two53(xs)) s_flag = 1;
                         if (seen == -1 && atomicCAS(&p.tag[x], -1, 0) == -1) {
                             st.vb += 1;
                             st.eb += (unsigned long long)deg;
-                        }
-                        uint64_t y = qm & need;
-                        while (y) {
-                            const int qq = __ffsll((long long)y) - 1;
-                            y &= y - 1;
-                            s_ql[qq] = seg;
                         }
                         if (deg <= pack_max) {
                             len = (int)deg;
@@ -594,10 +604,19 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     wa.sg[lane] = to_bits(xs);
                     const int total = __shfl_sync(kFull, incl, 31);
                     __syncwarp();
-                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, total, st.tight);
+                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, total, q.col, st.tight);
                     if (er) {
                         s_err = 1;
                         set_err(p.ctr, er);
+                    }
+                    // the query vertices among them (their mask has arrived by now)
+                    if (ok) {
+                        uint64_t y = qm & need;
+                        while (y) {
+                            const int qq = __ffsll((long long)y) - 1;
+                            y &= y - 1;
+                            s_ql[qq] = seg;
+                        }
                     }
                     __syncwarp();
                 }
@@ -623,7 +642,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                         wa.sg[0] = ((unsigned long long)(unsigned)ch.k << 32) | (unsigned)ch.e;
                     }
                     __syncwarp();
-                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, ch.na, st.tight);
+                    const int er = src_offers<PairT, kBits>(p, P, bk, s_cnt, s_done, tb, bcap, R, d, wa, ch.na, q.col, st.tight);
                     if (er) {
                         s_err = 1;
                         set_err(p.ctr, er);
@@ -653,20 +672,20 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             // ---------------- vertex scan, one query vertex r ----------------
             // delta_s.(r) = sigma_sr * sum over settled t with d(r, t) >= 1 and
             // d(s, r) + d(r, t) = d(s, t) of sigma_rt / sigma_st
-            const int r = p.vroot;
+            const int r = q.pos[p.vroot];
             unsigned long long dsr;
             typename PairT::Count ssr;
             P.get(r, dsr, ssr);
             double acc = 0.0;
             if (dsr != PairT::kUnreached && need) {
                 for (int e = tid; e < nh; e += bd) {
-                    const int t = hv[e];
-                    const unsigned long long rd = p.rdist[t];
+                    const int t = hv[e], tv = __ldg(q.inv + t);
+                    const unsigned long long rd = p.rdist[tv];
                     unsigned long long dt;
                     typename PairT::Count sst;
                     P.get(t, dt, sst);
                     if (rd == 0ull || rd >= dt || dsr + rd != dt) continue;
-                    acc += p.rsig[t] / (double)sst;
+                    acc += p.rsig[tv] / (double)sst;
                     st.pairs += 1;
                 }
             }
@@ -696,23 +715,28 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     cols |= 1ull << p.qcol[qq];
                 }
             }
-            for (int c = tid; c < 64; c += bd) s_cd[c] = ((cols >> c) & 1ull) ? P.dist(p.croot[c]) : PairT::kUnreached;
+            for (int c = tid; c < 64; c += bd) s_cd[c] = ((cols >> c) & 1ull) ? P.dist(q.pos[p.croot[c]]) : PairT::kUnreached;
             __syncthreads();
+            const int stride = wcols_stride(p.ncols);
             for (int e = tid; e < nh; e += bd) {
                 const int t = hv[e];
+                const size_t trow = (size_t)__ldg(q.inv + t) * stride;
                 unsigned long long dt;
                 typename PairT::Count sst;
                 P.get(t, dt, sst);
-                uint64_t y = cols;
-                while (y) {
-                    const int c = __ffsll((long long)y) - 1;
-                    y &= y - 1;
-                    const unsigned long long dc = s_cd[c];
-                    if (dc == PairT::kUnreached) continue;
-                    const unsigned long long rd = p.rdistq[(size_t)t * wcols_stride(p.ncols) + c];
-                    if (rd == 0ull || rd >= dt || dc + rd != dt) continue;
-                    atomicAdd(&s_msum[c], p.rsigq[(size_t)t * wcols_stride(p.ncols) + c] / (double)sst);
-                    st.pairs += 1;
+                // four columns (a sector of the row) per round of loads
+                for (int c0 = 0; c0 < stride; c0 += 4) {
+                    if (((cols >> c0) & 15ull) == 0ull) continue;
+                    const ulonglong2 ra = *reinterpret_cast<const ulonglong2 *>(p.rdistq + trow + c0);
+                    const ulonglong2 rb2 = *reinterpret_cast<const ulonglong2 *>(p.rdistq + trow + c0 + 2);
+                    const unsigned long long rd[4] = {ra.x, ra.y, rb2.x, rb2.y};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const unsigned long long dc = s_cd[c0 + k];  // unreached where the source needs no c
+                        if (dc == PairT::kUnreached || rd[k] == 0ull || rd[k] >= dt || dc + rd[k] != dt) continue;
+                        atomicAdd(&s_msum[c0 + k], p.rsigq[trow + c0 + k] / (double)sst);
+                        st.pairs += 1;
+                    }
                 }
             }
             __syncthreads();
@@ -724,7 +748,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     const int c = p.qcol[qq];
                     unsigned long long dcr;
                     typename PairT::Count scr;
-                    P.get(p.croot[c], dcr, scr);
+                    P.get(q.pos[p.croot[c]], dcr, scr);
                     s_dep[qq] = s_cd[c] != PairT::kUnreached ? (double)scr * s_msum[c] : 0.0;
                 }
             }
@@ -756,15 +780,16 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                     long long rb = 0, re = 0;
                     if (ok) {
                         v = hv[e0 + ii];
-                        rb = __ldg(p.off + v);
-                        re = __ldg(p.off + v + 1);
+                        const longlong2 row = __ldg(q.row + v);
+                        rb = row.x;
+                        re = row.y;
                     }
                     const bool shortrow = ok && re - rb <= pack_max;
                     double acc = 0.0;
-                    if (shortrow) acc = src_pull_c(p, ds, tb, dk, rb, re, rl, lpp);
+                    if (shortrow) acc = src_pull_c(p, q.col, ds, tb, dk, rb, re, rl, lpp);
                     acc = sum_lanes(acc, lpp);
                     if (shortrow && lead) {
-                        src_finalize(p, ds, need, s_dep, v, acc);
+                        src_finalize(p, q.inv, ds, need, s_dep, v, acc);
                         st.arcs += (unsigned long long)(re - rb);
                     } else if (ok && !shortrow && lead) {
                         const int nout = (int)((re - rb + CHB - 1) / CHB);
@@ -790,7 +815,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                 if (nch > 0) {
                     for (int c = warp; c < nch; c += nwarps) {
                         const Chunk ch = load_chunk(&chs[c]);
-                        const double v = sum_warp(src_pull_c(p, ds, tb, dk, ch.a0, ch.a0 + ch.na, lane, 32));
+                        const double v = sum_warp(src_pull_c(p, q.col, ds, tb, dk, ch.a0, ch.a0 + ch.na, lane, 32));
                         if (lane == 0) part[c] = v;
                         if (lane < ch.na) st.arcs += (unsigned long long)((ch.na - lane + 31) / 32);
                     }
@@ -800,7 +825,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
                         if (ch.k == 0) {
                             double acc = 0.0;
                             for (int k = 0; k < ch.nch; ++k) acc += part[c + k];
-                            src_finalize(p, ds, need, s_dep, ch.v, acc);
+                            src_finalize(p, q.inv, ds, need, s_dep, ch.v, acc);
                         }
                     }
                     __syncthreads();
@@ -815,7 +840,8 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             const int x = hv[e];
             P.clear(x);
             if (tb) {
-                const long long rb = __ldg(p.off + x), re = __ldg(p.off + x + 1);
+                const longlong2 row = __ldg(q.row + x);
+                const long long rb = row.x, re = row.y;
                 if (re > rb)
                     for (long long w = rb >> 5; w <= (re - 1) >> 5; ++w) tb[w] = 0u;
             }
@@ -926,6 +952,109 @@ bc_status clear_src_pairs(bc_graph *g, int layout) {
     return BC_OK;
 }
 
+void free_src_order(bcd_workspace &ws) {
+    dev_free(ws.spos);
+    dev_free(ws.sinv);
+    dev_free(ws.srow);
+    dev_free(ws.scol);
+}
+
+// Position classes: 0 for in-degrees of 2^31 and more, ... 31 for 1, 32 for 0.
+__device__ __forceinline__ int degree_class(const int64_t *roff, int v) {
+    const long long d = roff[v + 1] - roff[v];
+    return d == 0 ? 32 : d >= (1ll << 31) ? 0 : 1 + __clz((int)d) - 1;
+}
+
+__global__ void class_counts(const int64_t *roff, int32_t n, unsigned *cnt) {
+    __shared__ unsigned s_cnt[33];
+    if (threadIdx.x < 33) s_cnt[threadIdx.x] = 0u;
+    __syncthreads();
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+        atomicAdd(&s_cnt[degree_class(roff, v)], 1u);
+    __syncthreads();
+    if (threadIdx.x < 33 && s_cnt[threadIdx.x]) atomicAdd(&cnt[threadIdx.x], s_cnt[threadIdx.x]);
+}
+
+// One block: the classes' first positions.
+__global__ void class_starts(unsigned *cnt) {
+    if (threadIdx.x == 0) {
+        unsigned run = 0;
+        for (int c = 0; c < 33; ++c) {
+            const unsigned k = cnt[c];
+            cnt[c] = run;
+            run += k;
+        }
+    }
+}
+
+// Positions, a block's vertices of a class side by side.
+__global__ void assign_positions(const int64_t *off, const int64_t *roff, int32_t n, unsigned *next, int32_t *pos,
+                                 int32_t *inv, longlong2 *row) {
+    __shared__ unsigned s_cnt[33], s_at[33];
+    for (int v0 = blockIdx.x * blockDim.x; v0 < n; v0 += gridDim.x * blockDim.x) {
+        const int v = v0 + threadIdx.x;
+        if (threadIdx.x < 33) s_cnt[threadIdx.x] = 0u;
+        __syncthreads();
+        int c = 0;
+        unsigned rank = 0;
+        if (v < n) {
+            c = degree_class(roff, v);
+            rank = atomicAdd(&s_cnt[c], 1u);
+        }
+        __syncthreads();
+        if (threadIdx.x < 33 && s_cnt[threadIdx.x]) s_at[threadIdx.x] = atomicAdd(&next[threadIdx.x], s_cnt[threadIdx.x]);
+        __syncthreads();
+        if (v < n) {
+            const int x = (int)(s_at[c] + rank);
+            pos[v] = x;
+            inv[x] = v;
+            row[x] = make_longlong2(off[v], off[v + 1]);
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void heads_to_positions(const int32_t *col, int64_t m, const int32_t *pos, int32_t *out) {
+    for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x)
+        out[a] = pos[col[a]];
+}
+
+// The vertices' positions and the arrays that go with them, once per graph
+// (R-MAT 20: about half a millisecond).
+bc_status src_order(bc_graph *g) {
+    bcd_workspace &ws = g->ws;
+    if (ws.spos) return BC_OK;
+    const size_t n = (size_t)g->n;
+    unsigned *cnt = nullptr;
+    bc_status st;
+    if ((st = dev_alloc(&ws.sinv, n)) || (st = dev_alloc(&ws.srow, 2 * n)) ||
+        (st = dev_alloc(&ws.scol, (size_t)g->m)) || (st = dev_alloc(&cnt, 33)) || (st = dev_alloc(&ws.spos, n))) {
+        dev_free(cnt);
+        free_src_order(ws);
+        return st;
+    }
+    const unsigned blocks = (unsigned)std::max(1, g->num_sms * 4);
+    cudaMemsetAsync(cnt, 0, 33 * sizeof(unsigned), g->stream);
+    class_counts<<<blocks, 256, 0, g->stream>>>(g->d_roff, g->n, cnt);
+    class_starts<<<1, 32, 0, g->stream>>>(cnt);
+    assign_positions<<<blocks, 256, 0, g->stream>>>(g->d_off, g->d_roff, g->n, cnt, ws.spos, ws.sinv,
+                                                    reinterpret_cast<longlong2 *>(ws.srow));
+    if (g->m) heads_to_positions<<<blocks, 256, 0, g->stream>>>(g->d_col, g->m, ws.spos, ws.scol);
+    g->launches += 4;
+    cudaError_t e = cudaGetLastError();
+    // where the class before the last ended: the last one has no in-arcs
+    unsigned at[33] = {0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(at, cnt, sizeof(at), cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    ws.sheads = (int32_t)at[31];
+    dev_free(cnt);
+    if (e != cudaSuccess) {
+        free_src_order(ws);
+        return cuda_error(e, "source kernel order");
+    }
+    return BC_OK;
+}
+
 void free_src_arrays(bcd_workspace &ws) {
     dev_free(ws.sds);
     dev_free(ws.stb);
@@ -983,6 +1112,7 @@ bc_status grow_buf(T **p, int64_t *cap, int64_t need) {
 void free_src_state(bc_graph *g) {
     bcd_workspace &ws = g->ws;
     free_src_arrays(ws);
+    free_src_order(ws);
     dev_free(ws.sdep);
     dev_free(ws.sflag);
     dev_free(ws.snext);
@@ -1003,13 +1133,14 @@ bool src_kernel_applies(const bc_graph *g, const TravParams &p) {
 bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsigned long long *edges_out) {
     bcd_workspace &ws = g->ws;
     BCD_TRY(ensure_weighted_state(g));  // ring size, tag array
+    BCD_TRY(src_order(g));
     const int threads = src_threads(g->n);
     const int S = 64 * W;
     const int64_t nsrc = p.ntiles * S;
     const int R = ws.ring;
     // the settled bits join the staging and counters in shared memory while they fit
     const size_t ring = sizeof(WarpArcs) * (size_t)(threads / 32) + sizeof(uint32_t) * 2 * (size_t)R;
-    const size_t done = sizeof(uint32_t) * (((size_t)g->n + 31) / 32);
+    const size_t done = sizeof(uint32_t) * (((size_t)ws.sheads + 31) / 32);
     const bool bits = ring + done <= kSrcDynSmem;
     const size_t smem = ring + (bits ? done : 0);
     const void *wide = bits ? (const void *)wsrc_kernel<WidePairs, true> : (const void *)wsrc_kernel<WidePairs, false>;
@@ -1079,6 +1210,11 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
         q.sdep = ws.sdep;
         q.sflag = ws.sflag;
         q.next = ws.snext;
+        q.col = ws.scol;
+        q.row = reinterpret_cast<const longlong2 *>(ws.srow);
+        q.pos = ws.spos;
+        q.inv = ws.sinv;
+        q.heads = ws.sheads;
         q.n = g->n;
         q.bcap = ws.sbcap;
         q.chcap = ws.schcap;
