@@ -101,6 +101,9 @@ __host__ __device__ inline bool scan_too_long(unsigned long long terms, unsigned
     return terms > kScanAlways && terms * kScanPairCost > tight;
 }
 
+// Path counts below this have their inverses in a table.
+constexpr int kInverses = 2048;
+
 struct TravParams {
     int32_t n;
     int32_t mode;
@@ -114,6 +117,7 @@ struct TravParams {
     int32_t pad0;
     int32_t *tag;       // [n] last level a vertex was appended at, -1 none
     double *sigma;      // [n * S] sigma (unweighted: 32-bit counts, or fp64 after an overflow; weighted: then c in place)
+    const double *inv;  // [kInverses] 1 / k (k = 0: 1), unweighted
     double *acc;        // [n * S] backward sums of c over tight out-arcs (unweighted), zero between levels
     // level history
     int32_t *hv;        // [hcap]
@@ -212,6 +216,7 @@ struct TravParams {
 struct bcd_workspace {
     int W = 0;           // mask words per tile (S = 64 W sources)
     int teams = 1;       // tiles whose state is held at once (unweighted): the arrays of state below hold that many
+    bool teams_ready = false;  // that number is the graph's (teams_for)
     int64_t n = 0;
     int64_t m = 0;
     // dense state
@@ -219,6 +224,7 @@ struct bcd_workspace {
     int vs_stride = 0;
     int32_t *tag = nullptr;
     double *sigma = nullptr;
+    double *inv = nullptr;        // [kInverses] 1 / k (unweighted graphs)
     size_t sigma_bytes = 8;       // bytes per count (4: 32-bit counts of unweighted graphs)
     bool sigma_zero = false;      // the slab is all zero
     int64_t sigma_key = -1;       // unweighted: row width, count type and chunk_arcs the slab was last used with
@@ -355,6 +361,7 @@ struct bc_graph {
     int pull_permille = 0;        // bottom-up levels: frontier out-arcs >= pull_permille / 1000 of m (0: never)
     int wshort = 32;              // weighted kernel: longest row one lane walks alone
     int weighted_kernel = 2;      // weighted graphs: 1 tile kernel, 2 one source per block
+    bool queried = false;         // the handle has been asked for more than reach sets
     bcd_workspace ws;
     int64_t launches = 0;
     int last_grid = 0;                       // blocks of the last traversal launch

@@ -135,6 +135,13 @@ __global__ void fill_i32(int32_t *p, int64_t cnt, int32_t val) {
         p[i] = val;
 }
 
+// The table of 1 / k: computed once, since a block's own 2,048 fp64 divisions
+// would take longer than loading it (8 us per launch on the few fp64 units).
+__global__ void fill_inverses(double *inv) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    inv[k] = 1.0 / (double)(k > 0 ? k : 1);
+}
+
 __global__ void positions(const int32_t *list, int64_t cnt, int32_t *pos) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (long long)gridDim.x * blockDim.x)
         pos[list[i]] = (int32_t)i;
@@ -330,6 +337,7 @@ void free_workspace(bc_graph *g) {
     dev_free(ws.vs);
     dev_free(ws.tag);
     dev_free(ws.sigma);
+    dev_free(ws.inv);
     dev_free(ws.acc);
     dev_free(ws.hv);
     dev_free(ws.hm);
@@ -418,6 +426,50 @@ static int teams_for(int64_t n, int64_t m, int W) {
     return t;
 }
 
+// The small arrays that every team has its own part of.
+static bc_status alloc_team_state(bc_graph *g) {
+    bcd_workspace &ws = g->ws;
+    const size_t t = (size_t)ws.teams, n = (size_t)ws.n, S = 64 * (size_t)ws.W;
+    dev_free(ws.vs);
+    dev_free(ws.tag);
+    dev_free(ws.qlevel);
+    dev_free(ws.dep);
+    dev_free(ws.vsum);
+    dev_free(ws.msum);
+    dev_free(ws.srcflag);
+    dev_free(ws.ctr);
+    BCD_TRY(dev_alloc(&ws.vs, t * n * ws.vs_stride));
+    BCD_TRY(dev_alloc(&ws.tag, t * n));
+    BCD_TRY(dev_alloc(&ws.qlevel, t * S * 64));
+    BCD_TRY(dev_alloc(&ws.dep, t * S * 64));
+    BCD_TRY(dev_alloc(&ws.vsum, t * 2 * S));
+    BCD_TRY(dev_alloc(&ws.msum, t * 2 * S * 64));
+    BCD_TRY(dev_alloc(&ws.srcflag, t * std::max<size_t>(ws.W, 4)));
+    BCD_TRY(dev_alloc((char **)&ws.ctr, kCounterBytes + sizeof(TeamBar) * t));
+    return BC_OK;
+}
+
+// State for as many teams as a call of several tiles runs at once, where the
+// workspace was built for reach sets. Callers take the arrays' addresses after
+// this.
+static bc_status ensure_teams(bc_graph *g, int64_t ntiles) {
+    bcd_workspace &ws = g->ws;
+    if (g->weighted || ntiles < 2 || ws.teams_ready) return BC_OK;
+    ws.teams_ready = true;
+    const int t = teams_for(ws.n, ws.m, ws.W);
+    if (t <= ws.teams) return BC_OK;
+    ws.teams = t;
+    dev_free(ws.sigma);  // prepare_slabs allocates these for the new count
+    dev_free(ws.acc);
+    ws.sigma_key = -1;
+    bc_status st = alloc_team_state(g);
+    if (st == BC_OK) st = alloc_history(g, ws.hcap, ws.ccap, ws.pcap, ws.hmcap);
+    if (st == BC_OK) st = alloc_levels(g, ws.maxlev);
+    if (st == BC_OK) st = reset_dense_state(g);
+    if (st != BC_OK) free_workspace(g);
+    return st;
+}
+
 static bc_status build_workspace(bc_graph *g, int W) {
     bcd_workspace &ws = g->ws;
     free_workspace(g);
@@ -427,14 +479,19 @@ static bc_status build_workspace(bc_graph *g, int W) {
     ws.m = m;
     // the weighted kernel keeps no masks; the one-word reach traversals do
     ws.vs_stride = g->weighted ? 4 : ((3 * W + 3) / 4) * 4;
-    ws.teams = g->weighted ? 1 : teams_for(n, m, W);
-    const size_t t = (size_t)ws.teams;
-    BCD_TRY(dev_alloc(&ws.vs, t * n * ws.vs_stride));
-    BCD_TRY(dev_alloc(&ws.tag, t * n));
-    // counts of unweighted graphs: 32 bits until a launch needs fp64; the
-    // accumulators of Eq. 4 come with the first launch that needs them
-    ws.sigma_bytes = g->weighted ? sizeof(double) : sizeof(uint32_t);
-    BCD_TRY(dev_alloc(&ws.sigma, t * n * 64 * W * ws.sigma_bytes / sizeof(double)));
+    // a handle that only asks for reach sets keeps one tile's state
+    // (ensure_teams); the counts of unweighted graphs and the accumulators of
+    // Eq. 4 come with the first launch that needs them
+    ws.teams_ready = g->queried;
+    ws.teams = g->queried && !g->weighted ? teams_for(n, m, W) : 1;
+    BCD_TRY(alloc_team_state(g));
+    if (g->weighted) {
+        BCD_TRY(dev_alloc(&ws.sigma, (size_t)n * 64 * W));
+    } else {
+        BCD_TRY(dev_alloc(&ws.inv, (size_t)kInverses));
+        fill_inverses<<<kInverses / 256, 256, 0, g->stream>>>(ws.inv);
+        BCD_CUDA(cudaGetLastError());
+    }
     const int64_t ch = g->chunk_arcs;
     BCD_TRY(alloc_history(g, 8 * n + 4096, 8 * n + 8 * (m / ch) + 4096, 8 * (m / ch) + 4096, 16 * n + 4096));
     BCD_TRY(alloc_levels(g, std::min<int64_t>(g->weighted ? std::max<int64_t>(n + 1, 65536) : n + 1,
@@ -446,20 +503,14 @@ static bc_status build_workspace(bc_graph *g, int W) {
     BCD_TRY(dev_alloc(&ws.hublev, (size_t)n));
     ws.hub = -1;
     BCD_TRY(dev_alloc(&ws.dlist, (size_t)n + 64 * (size_t)W + 256));  // union padded to whole tiles
-    BCD_TRY(dev_alloc(&ws.qlevel, t * 64 * W * 64));
-    BCD_TRY(dev_alloc(&ws.dep, t * 64 * W * 64));
     // vertex scan state
     if (g->weighted)
         BCD_TRY(dev_alloc(&ws.rdist, (size_t)n));
     else
         BCD_TRY(dev_alloc(&ws.rlev, (size_t)n));
     BCD_TRY(dev_alloc(&ws.rsig, (size_t)n));
-    BCD_TRY(dev_alloc(&ws.vsum, t * 2 * 64 * W));
-    BCD_TRY(dev_alloc(&ws.msum, t * 2 * 64 * W * 64));
     BCD_TRY(dev_alloc(&ws.rtile, (size_t)64 * W));
     BCD_TRY(dev_alloc(&ws.qflags, 64));
-    BCD_TRY(dev_alloc(&ws.srcflag, t * std::max(W, 4)));
-    BCD_TRY(dev_alloc((char **)&ws.ctr, kCounterBytes + sizeof(TeamBar) * t));
     ws.scratch_len = scan_scratch_len(n) + 64;
     BCD_TRY(dev_alloc(&ws.scratch64, (size_t)ws.scratch_len + 256));
     BCD_TRY(dev_alloc(&ws.small, (size_t)kSmallWords));
@@ -467,7 +518,7 @@ static bc_status build_workspace(bc_graph *g, int W) {
     BCD_CUDA(cudaMemsetAsync(ws.rvmask, 0, sizeof(uint64_t) * (size_t)n, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.need, 0, sizeof(uint64_t) * (size_t)n, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.qmask, 0, sizeof(uint64_t) * (size_t)n, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.dep, 0, sizeof(double) * t * 64 * W * 64, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.dep, 0, sizeof(double) * 64 * W * 64, g->stream));
     BCD_CUDA(cudaMallocHost(&ws.pinned, 1 << 20));
     ws.pinned_cap = 1 << 20;
     return BC_OK;
@@ -741,6 +792,17 @@ static bool use_vertex_scan(const bc_graph *g, size_t nroots) {
     return g->accumulation >= 3 && nroots <= 64;
 }
 
+// Whether the scan's terms of an unweighted group are worth counting before it
+// is tried: a query vertex of in-degree x out-degree 64 times the mean's square
+// may have a large share of all shortest paths run through it.
+static bool scan_on_trial(const bc_graph *g, const std::vector<int32_t> &roots) {
+    if (g->weighted) return false;
+    const double mean = (double)g->m / (double)g->n;
+    for (int32_t r : roots)
+        if ((double)(g->h_off[r + 1] - g->h_off[r]) * (double)(g->h_roff[r + 1] - g->h_roff[r]) >= 64.0 * mean * mean) return true;
+    return false;
+}
+
 // Offsets in bcd_workspace::small of the column tables of a multi-vertex scan.
 constexpr int kSmallQcol = 1024;   // 64 int32: column of each query bit
 constexpr int kSmallCroot = 1056;  // 64 int32: vertex of each column
@@ -980,6 +1042,7 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
     std::vector<uint32_t> qflags(64, 0);
     int levels = 0;
     unsigned long long edges = 0;
+    BCD_TRY(ensure_teams(g, nrun));
     const bool scan = nrun > 0 && use_vertex_scan(g, roots.size());
     const bool multi = scan && roots.size() >= 2;
     if (scan) {
@@ -1051,16 +1114,18 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
             return BC_OK;
         };
         std::vector<uint32_t> cal_flags(64, 0);
-        if (multi && g->accumulation == 4 && (nrun > 1 || !g->weighted)) {
+        const bool trial = multi && g->accumulation == 4 && scan_on_trial(g, roots);
+        if (multi && g->accumulation == 4 && (nrun > 1 || trial)) {
             // choose the backward on the group's first tile: the scan's terms
             // (a division and a shared-memory add each) against the push's
             // tight (source, arc) pairs (an fp64 reduction each), at the
-            // measured cost ratio of about 16. Unweighted: the terms are
-            // counted before any is added, and a tile with too many of them is
+            // measured cost ratio of about 16. With a hub among the query
+            // vertices of an unweighted graph the terms are counted before any
+            // is added, and a tile with too many of them is
             // left to the push (R-MAT 20 with hubs among the query vertices: 373
             // million terms took 70 ms on the one tile, counting them and
             // repeating its forward pass 5 ms).
-            BCD_TRY(launch_tiles(true, 0, 1, !g->weighted));
+            BCD_TRY(launch_tiles(true, 0, 1, trial));
             if (g->last.scan_skipped) {
                 BCD_TRY(launch_tiles(false, 0, nrun));
             } else {
@@ -1230,6 +1295,7 @@ bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::ve
     const int S = 64 * W;
     const int64_t ntiles = (int64_t)srcs.size() / S;
     if (ntiles * S != (int64_t)srcs.size() || ntiles == 0) return set_error(BC_E_INTERNAL, "run_slice: ragged slice");
+    BCD_TRY(ensure_teams(g, ntiles));
     std::vector<int32_t> vs;
     std::vector<uint64_t> ms;
     uint64_t used = 0;  // query slots some source of the slice serves
@@ -1308,8 +1374,9 @@ bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::ve
     };
     if (edges) *edges = 0;
     std::vector<uint32_t> cal_flags(64, 0);
-    if (multi && g->accumulation == 4 && (ntiles > 1 || !g->weighted)) {
-        BCD_TRY(launch(true, 0, 1, !g->weighted));
+    const bool trial = multi && g->accumulation == 4 && scan_on_trial(g, roots);
+    if (multi && g->accumulation == 4 && (ntiles > 1 || trial)) {
+        BCD_TRY(launch(true, 0, 1, trial));
         if (g->last.scan_skipped) {
             BCD_TRY(launch(false, 0, ntiles));
         } else {
@@ -1347,6 +1414,7 @@ void begin_call(bc_graph *g) {
 bc_status check_graph(bc_graph *g, const char *fn) {
     if (!g) return set_error(BC_E_INVALID_ARG, std::string(fn) + ": NULL graph");
     begin_call(g);
+    g->queried = true;
     BCD_TRY(ensure_workspace(g, tile_words_of(g)));
     if (g->weighted) BCD_TRY(ensure_weighted_state(g));
     return BC_OK;

@@ -697,7 +697,6 @@ __device__ __noinline__ void gather_level(int L, long long ics, long long iccnt,
 // 1 / sigma. The chip's fp64 units are few (a warp instruction holds an SM's
 // for 16 cycles, so the dozen of a division cost more than the rest of a
 // step): counts up to kInverses, nearly all of them, are looked up.
-constexpr int kInverses = 2048;
 __device__ __forceinline__ double *inverses() {
     __shared__ double s_inv[kInverses];
     return s_inv;
@@ -1389,7 +1388,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
     __shared__ int32_t s_lstop;
     double *const s_inv = inverses();  // 1 / k
     if (MODE != kModeReach && sizeof(T) == 4)
-        for (int i = threadIdx.x; i < kInverses; i += blockDim.x) s_inv[i] = 1.0 / (double)max(i, 1);
+        for (int i = threadIdx.x; i < kInverses; i += blockDim.x) s_inv[i] = p.inv[i];
     const bool timer = team == 0 && leader;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
     unsigned long long ns_fwd = 0, ns_bwd = 0, ns_other = 0;
@@ -1752,11 +1751,11 @@ bc_status prepare_slabs(bc_graph *g, int W, bool eq4) {
     bcd_workspace &ws = g->ws;
     const size_t pairs = (size_t)ws.teams * (size_t)ws.n * 64 * (size_t)ws.W;
     const size_t bytes = ws.swide ? sizeof(double) : sizeof(uint32_t);
-    if (ws.sigma_bytes < bytes) {
+    if (!ws.sigma || ws.sigma_bytes < bytes) {
         dev_free(ws.sigma);
         ws.sigma_key = -1;
         ws.sigma_zero = false;
-        const bc_status st = dev_alloc(&ws.sigma, pairs);
+        const bc_status st = dev_alloc(&ws.sigma, pairs * bytes / sizeof(double));
         if (st != BC_OK) {
             free_workspace(g);
             return st;
@@ -1787,8 +1786,10 @@ bc_status reset_dense_state(bc_graph *g) {
     const size_t t = (size_t)ws.teams, n = (size_t)ws.n, lev = (size_t)(ws.maxlev + 2);
     BCD_CUDA(cudaMemsetAsync(ws.vs, 0, sizeof(uint64_t) * t * n * ws.vs_stride, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.tag, 0xff, sizeof(int32_t) * t * n, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.sigma, 0, ws.sigma_bytes * t * n * 64 * ws.W, g->stream));
-    ws.sigma_zero = true;
+    if (ws.sigma) {
+        BCD_CUDA(cudaMemsetAsync(ws.sigma, 0, ws.sigma_bytes * t * n * 64 * ws.W, g->stream));
+        ws.sigma_zero = true;
+    }
     BCD_CUDA(cudaMemsetAsync(ws.lev_cnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.lev_ccnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.lev_grab, 0, sizeof(unsigned long long) * t * 6 * lev, g->stream));
@@ -1810,6 +1811,7 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         p.tag = ws.tag;
         p.sigma = ws.sigma;
         p.acc = ws.acc;
+        p.inv = ws.inv;
         p.roff = g->d_roff;  // R(G): in-arcs for the backward push and the weighted sigma pull
         p.rcol = g->d_rcol;
         p.hv = ws.hv;

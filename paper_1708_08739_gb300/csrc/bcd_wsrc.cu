@@ -1134,7 +1134,11 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     bcd_workspace &ws = g->ws;
     BCD_TRY(ensure_weighted_state(g));  // ring size, tag array
     BCD_TRY(src_order(g));
-    const int threads = src_threads(g->n);
+    // blocks by the size of the graph (state is held for that many); a launch
+    // with fewer sources than that takes wider ones
+    const int base_threads = src_threads(g->n);
+    int threads = base_threads;
+    while (threads < kSrcThreads && (int64_t)g->num_sms * (kSrcThreads / (2 * threads)) >= p.ntiles * 64 * W) threads *= 2;
     const int S = 64 * W;
     const int64_t nsrc = p.ntiles * S;
     const int R = ws.ring;
@@ -1155,15 +1159,15 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     if (ws.sbcap == 0) {
         // queued vertices of one distance of one source: a few times the
         // average vertices per distance value, and at least 2^21 entries
-        // over the whole ring (8 MB), or 32 per vertex; grown on overflow
-        const int64_t whole = std::min<int64_t>((int64_t)1 << 21, 32 * (int64_t)g->n);
+        // over the whole ring (8 MB), or 16 per vertex; grown on overflow
+        const int64_t whole = std::min<int64_t>((int64_t)1 << 21, 16 * (int64_t)g->n);
         int64_t b = 64;
         while ((b < 4 * (int64_t)g->n / R || b * R < whole) && b < ((int64_t)1 << 30)) b *= 2;
         ws.sbcap = b;
         ws.schcap = 16384;
         ws.smaxlev = 8192;
     }
-    int blocks = g->num_sms * per_sm;
+    int blocks = g->num_sms * per_sm * (threads / base_threads);
     {
         size_t fr = 0, tot = 0;
         BCD_CUDA(cudaMemGetInfo(&fr, &tot));
@@ -1173,7 +1177,7 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
         blocks = (int)std::min<size_t>((size_t)blocks, budget / per);
         if (blocks < 1) return set_error(BC_E_OOM, "weighted source kernel: no room for one block's state");
     }
-    if (ws.sblocks != blocks || !ws.sds) {
+    if (ws.sblocks < blocks || !ws.sds) {
         const bc_status st = alloc_src_arrays(g, blocks);
         if (st != BC_OK) {
             free_src_arrays(ws);
@@ -1231,10 +1235,10 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
         const bool timed = cudaEventCreate(&ev0) == cudaSuccess && cudaEventCreate(&ev1) == cudaSuccess;
         if (timed) cudaEventRecord(ev0, g->stream);
         void *args[] = {(void *)&p, (void *)&q};
-        const cudaError_t le = cudaLaunchKernel(layout == 2 ? narrow : wide, dim3((unsigned)ws.sblocks),
+        const cudaError_t le = cudaLaunchKernel(layout == 2 ? narrow : wide, dim3((unsigned)std::min(ws.sblocks, g->num_sms * per_sm)),
                                                 dim3((unsigned)threads), args, smem, g->stream);
         g->launches += 1;
-        g->last_grid = ws.sblocks;
+        g->last_grid = std::min(ws.sblocks, g->num_sms * per_sm);
         if (le != cudaSuccess) {
             if (timed) {
                 cudaEventDestroy(ev0);
