@@ -276,17 +276,16 @@ def solve_step(bcd, dg, specs, rank, world, dist):
 def algorithmic_bytes(info, weighted=False):
     """The traversal's algorithmic bytes (see the design notes): graph
     structure 2 (8 |V_B| + 4 |E_B|) summed over tiles (8 bytes per arc with
-    its weight); the forward pass, 24 bytes per reached (source, vertex) pair
-    (level and sigma written and read back; 32 with 8-byte distances) and 8
-    per tight (source, arc) pair (sigma of the tail); the Eq. 4 backward, on
-    the tiles that ran it, 16 more per reached pair (delta written and read)
-    and 16 per tight pair (sigma and delta of the head); the vertex scan, 16
-    per term (sigma_st and sigma_rt)."""
-    arc = 8.0 if weighted else 4.0
-    pair = 32.0 if weighted else 24.0
+    its weight); the forward pass, 16 bytes per reached (source, vertex) pair
+    (level and 4-byte count written and read back; 32 with 8-byte distances
+    and counts) and 4 (8) per tight (source, arc) pair (the tail's count); the
+    Eq. 4 backward, on the tiles that ran it, 16 more per reached pair (the
+    accumulator written and read) and 16 per tight pair (its update); the
+    vertex scan, 12 (16) per term (sigma_st and sigma_rt)."""
+    arc, pair, tight, term = (8.0, 32.0, 8.0, 16.0) if weighted else (4.0, 16.0, 4.0, 12.0)
     return (2.0 * (8.0 * info["union_vertices"] + arc * info["union_arcs"]) + pair * info["reached_pairs"] +
-            8.0 * info["tight_pairs"] + 16.0 * info["eq4_reached_pairs"] + 16.0 * info["eq4_tight_pairs"] +
-            16.0 * info["scan_pairs"])
+            tight * info["tight_pairs"] + 16.0 * info["eq4_reached_pairs"] + 16.0 * info["eq4_tight_pairs"] +
+            term * info["scan_pairs"])
 
 
 def run_gpu(args):

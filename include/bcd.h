@@ -374,7 +374,9 @@ void bc_server_destroy(bc_server *srv);
  *                  the columns of the queries that need the source;
  *                  4 (default) 2 for one-vertex groups and, for a group
  *                  at several vertices, 3 on its
- *                  first tile, then for the remaining tiles the scan when
+ *                  first tile (unless, on an unweighted graph with a hub
+ *                  among the vertices, that tile's terms, counted first, are
+ *                  above 2^23 and too many by the rule that follows), then for the remaining tiles the scan when
  *                  its terms on that tile, weighted 16 to 1, did not
  *                  outnumber the tight (source, arc) pairs the Eq. 4 push
  *                  would add, else 1. The scan wins where few shortest
@@ -392,13 +394,14 @@ void bc_server_destroy(bc_server *srv);
  *                  arc), the others top-down (the frontier pushes sigma
  *                  along its out-arcs); 1..1000, or -1 for top-down only.
  *                  Results are identical either way (sigma sums integers).
- *   weighted_short_row  weighted kernels: a settled vertex (source kernel:
- *                  whose out-row; tile kernel: a (vertex, source) pair whose
- *                  in- and out-rows both) has at most this many arcs is
- *                  handled by the lanes given to it in its level (1 to 32,
- *                  tile kernel 1 to 8); longer rows are cut into chunk_arcs
- *                  chunks that a warp takes with lanes over arcs (1..1024,
- *                  default 32).
+ *   weighted_short_row  weighted kernels, 1..1024 (default 32). Source kernel:
+ *                  settled vertices whose out-rows have at most four times
+ *                  this many arcs are packed together onto a warp's lanes;
+ *                  tile kernel: a (vertex, source) pair whose in- and
+ *                  out-rows both have at most this many arcs is handled by
+ *                  the lanes given to it in its level (1 to 8). Longer rows
+ *                  are cut into chunk_arcs chunks that a warp takes with
+ *                  lanes over arcs.
  *   timeout_us     limit, in microseconds of wall time, on every wait of a
  *                  traversal kernel at a grid-wide barrier (default
  *                  10,000,000: 10 s), and on the time one block of the
