@@ -310,7 +310,10 @@ __device__ __forceinline__ int src_offers(const TravParams &p, const PairT &P, u
         for (int j = 0; j < kLanesBatch; ++j) {
             if (y[j] < 0) continue;
             const unsigned long long nd = d + w[j];
-            if (nd > PairT::dist_of(cur[j])) continue;
+            const unsigned long long cd = PairT::dist_of(cur[j]);
+            // an unreached head takes every offer, also one past the narrow
+            // layout's distances, for which the launch reruns
+            if (nd > cd && cd != PairT::kUnreached) continue;
             const int v = (int)(vs >> (5 * j)) & 31;
             const int r = P.offer(y[j], nd, from_bits<typename PairT::Count>(wa.sg[v]), cur[j]);
             if (r > 0) {
