@@ -1802,8 +1802,12 @@ bc_status reset_dense_state(bc_graph *g) {
     return BC_OK;
 }
 
+// Reruns after an overflow have no count of their own: each one enlarges what
+// was full, up to a limit at which the growing function returns BC_E_OOM, or
+// takes the one step to fp64 counts. (A tile of 256 sources on a path doubles
+// its history five times, and may meet a wide count besides.)
 bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsigned long long *edges_out) {
-    for (int attempt = 0; attempt < 6; ++attempt) {
+    for (;;) {
         bcd_workspace &ws = g->ws;
         if (!g->weighted && p.mode != kModeReach) BCD_TRY(prepare_slabs(g, W, p.mode == kModeSpd));
         p.vs = ws.vs;
@@ -1912,8 +1916,9 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         }
         if (c.err == kDevWide) {
             // a path count of 2^26: fp64 counts from now on
-            ws.swide = true;
             BCD_TRY(reset_dense_state(g));
+            if (ws.swide) return set_error(BC_E_INTERNAL, "traversal: fp64 counts asked for a wider form");
+            ws.swide = true;
             if (p.qflags) BCD_CUDA(cudaMemsetAsync(p.qflags, 0, sizeof(uint32_t) * 64, g->stream));
             continue;
         }
@@ -1938,7 +1943,6 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
             BCD_CUDA(cudaMemsetAsync(p.rvmask, 0, sizeof(uint64_t) * (size_t)g->n, g->stream));
         if (p.qflags) BCD_CUDA(cudaMemsetAsync(p.qflags, 0, sizeof(uint32_t) * 64, g->stream));
     }
-    return set_error(BC_E_OOM, "traversal: level history did not fit after growing it");
 }
 
 }  // namespace bcd

@@ -1190,7 +1190,7 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     BCD_TRY(grow_buf(&ws.sdep, &ws.sdep_cap, nsrc * 64));
     BCD_TRY(grow_buf(&ws.sflag, &ws.sflag_cap, nsrc));
     if (!ws.snext) BCD_TRY(dev_alloc(&ws.snext, 1));
-    for (int attempt = 0; attempt < 8; ++attempt) {
+    for (;;) {  // each rerun enlarges what was full, up to its limit, or takes the one step to wide pairs
         p.off = g->d_off;
         p.col = g->d_col;
         p.wt = g->d_w;
@@ -1285,6 +1285,7 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
         if (c.err == kDevCancelled) return set_error(BC_E_CANCELLED, "traversal: cancelled by bc_cancel");
         if (c.err == kDevWide) {
             // a count of 2^40 or a distance of 2^24 - 1: 16-byte pairs from now on
+            if (layout == 1) return set_error(BC_E_INTERNAL, "weighted source kernel: wide pairs asked for a wider form");
             ws.swide = true;
             continue;
         }
@@ -1316,7 +1317,6 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
             return st;
         }
     }
-    return set_error(BC_E_OOM, "weighted source kernel: state did not fit after growing it");
 }
 
 }  // namespace bcd
