@@ -5,6 +5,7 @@ bit-exact against the oracle."""
 import numpy as np
 import pytest
 
+import graphgen as gg
 import oracle as O
 from helpers import csr
 
@@ -36,3 +37,25 @@ def test_noalloc_edges(n, row):
         k = bcd.bc_rv_compute_noalloc(roff.data_ptr(), rcol.data_ptr(), n, r, out.data_ptr(), n,
                                       torch.cuda.current_stream().cuda_stream)
         assert k == want.shape[0] and np.array_equal(out[:k].cpu().numpy(), want), (n, row, r)
+
+
+def device_csr(og):
+    torch = pytest.importorskip("torch")
+    roff, rcol = torch.from_numpy(og.roff.copy()).cuda(), torch.from_numpy(og.rcol.copy()).cuda()
+    return roff, rcol if rcol.numel() else torch.zeros(1, dtype=torch.int32, device="cuda")
+
+
+@pytest.mark.parametrize("n,deg", [(300, 150), (2048, 127), (2048, 129), (4096, 500), (9001, 300)])
+def test_noalloc_dense(n, deg):
+    """Graphs whose arcs, not their vertices, decide how many blocks run."""
+    torch = pytest.importorskip("torch")
+    import paper_1708_08739_gb300 as bcd
+    g = gg.erdos_renyi(n, n * deg, 5)
+    og = O.Graph.from_csr(g)
+    roff, rcol = device_csr(og)
+    out = torch.full((n + 1,), -7, dtype=torch.int32, device="cuda")
+    for r in (0, n // 3, n - 1):
+        want = O.rv(og, r)
+        k = bcd.bc_rv_compute_noalloc(roff.data_ptr(), rcol.data_ptr(), n, r, out.data_ptr(), n,
+                                      torch.cuda.current_stream().cuda_stream)
+        assert k == want.shape[0] and np.array_equal(out[:k].cpu().numpy(), want), (n, r)
