@@ -216,7 +216,7 @@ struct TravParams {
 struct bcd_workspace {
     int W = 0;           // mask words per tile (S = 64 W sources)
     int teams = 1;       // tiles whose state is held at once (unweighted): the arrays of state below hold that many
-    bool teams_ready = false;  // that number is the graph's (teams_for)
+    bool teams_full = false;   // that number is the most for the graph (teams_for)
     int64_t n = 0;
     int64_t m = 0;
     // dense state
@@ -361,7 +361,7 @@ struct bc_graph {
     int pull_permille = 0;        // bottom-up levels: frontier out-arcs >= pull_permille / 1000 of m (0: never)
     int wshort = 32;              // weighted kernel: longest row one lane walks alone
     int weighted_kernel = 2;      // weighted graphs: 1 tile kernel, 2 one source per block
-    bool queried = false;         // the handle has been asked for more than reach sets
+    int64_t tiles_ahead = 1;      // most tiles that a launch of the call now running can have
     bcd_workspace ws;
     int64_t launches = 0;
     int last_grid = 0;                       // blocks of the last traversal launch
@@ -430,7 +430,7 @@ bc_status set_query_bit(bc_graph *g, int32_t v, int bit, bool on);
 bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::vector<uint64_t> &needs,
                     const std::vector<uint32_t> &mult, uint64_t exact_q, const std::vector<int32_t> &slot_roots,
                     std::vector<double> &partials, uint32_t *qflags, unsigned long long *edges);
-bc_status check_graph(bc_graph *g, const char *fn);
+bc_status check_graph(bc_graph *g, const char *fn, int64_t tiles);
 void begin_call(bc_graph *g);
 bc_status prepare_ordering(bc_graph *g);
 // Tile order of a source: hop distance to the hub, then arcs two hops away (descending).

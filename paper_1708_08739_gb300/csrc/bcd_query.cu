@@ -450,12 +450,12 @@ static bc_status alloc_team_state(bc_graph *g) {
 }
 
 // State for as many teams as a call of several tiles runs at once, where the
-// workspace was built for reach sets. Callers take the arrays' addresses after
-// this.
+// workspace was built for a call of fewer tiles (a reach set, one tile). Callers
+// take the arrays' addresses after this.
 static bc_status ensure_teams(bc_graph *g, int64_t ntiles) {
     bcd_workspace &ws = g->ws;
-    if (g->weighted || ntiles < 2 || ws.teams_ready) return BC_OK;
-    ws.teams_ready = true;
+    if (g->weighted || ntiles <= ws.teams || ws.teams_full) return BC_OK;
+    ws.teams_full = true;
     const int t = teams_for(ws.n, ws.m, ws.W);
     if (t <= ws.teams) return BC_OK;
     ws.teams = t;
@@ -479,11 +479,14 @@ static bc_status build_workspace(bc_graph *g, int W) {
     ws.m = m;
     // the weighted kernel keeps no masks; the one-word reach traversals do
     ws.vs_stride = g->weighted ? 4 : ((3 * W + 3) / 4) * 4;
-    // a handle that only asks for reach sets keeps one tile's state
-    // (ensure_teams); the counts of unweighted graphs and the accumulators of
-    // Eq. 4 come with the first launch that needs them
-    ws.teams_ready = g->queried;
-    ws.teams = g->queried && !g->weighted ? teams_for(n, m, W) : 1;
+    // no more teams than the call can have tiles: a handle's first question is
+    // often one of few samples, and the arrays of 16 teams took 0.4 ms of it (45,000
+    // vertices; ensure_teams adds teams when a call has more tiles). The counts
+    // of unweighted graphs and the accumulators of Eq. 4 come with the first
+    // launch that needs them
+    const int full = g->weighted ? 1 : g->tiles_ahead > 1 ? teams_for(n, m, W) : INT32_MAX;
+    ws.teams = (int)std::min<int64_t>(full, std::max<int64_t>(1, g->tiles_ahead));
+    ws.teams_full = ws.teams == full;
     BCD_TRY(alloc_team_state(g));
     if (g->weighted) {
         BCD_TRY(dev_alloc(&ws.sigma, (size_t)n * 64 * W));
@@ -1409,12 +1412,14 @@ bc_status prepare_ordering(bc_graph *g) { return g->source_order == 1 ? ensure_h
 // A call starts: a cancel request left from before it is dropped.
 void begin_call(bc_graph *g) {
     if (g->cancel_h) __atomic_store_n(g->cancel_h, 0, __ATOMIC_SEQ_CST);
+    g->tiles_ahead = 1;
 }
 
-bc_status check_graph(bc_graph *g, const char *fn) {
+// ... one that runs at most `tiles` tiles in a launch.
+bc_status check_graph(bc_graph *g, const char *fn, int64_t tiles) {
     if (!g) return set_error(BC_E_INVALID_ARG, std::string(fn) + ": NULL graph");
     begin_call(g);
-    g->queried = true;
+    g->tiles_ahead = tiles;
     BCD_TRY(ensure_workspace(g, tile_words_of(g)));
     if (g->weighted) BCD_TRY(ensure_weighted_state(g));
     return BC_OK;
@@ -1426,7 +1431,16 @@ static bc_status run_batch(bc_graph *g, const bc_query *queries, int64_t nq, bc_
     if (nshards < 1 || shard < 0 || shard >= nshards)
         return set_error(BC_E_INVALID_ARG, "bc_batch_shard: need 0 <= shard < nshards");
     if (nq < 0 || (nq > 0 && (!queries || !out))) return set_error(BC_E_INVALID_ARG, "bc_batch: bad query array");
-    BCD_TRY(check_graph(g, "bc_batch"));
+    // at most every vertex, or as many sources as the queries draw
+    double most = 0.0;
+    for (int64_t i = 0; i < nq && most < (double)g->n; ++i) {
+        const bc_query &q = queries[i];
+        if (q.kind == BC_QUERY_EXACT) most += (double)g->n;
+        if (q.kind == BC_QUERY_APPROX && q.eps > 0.0 && q.delta > 0.0) most += samples_for(q.eps, q.delta);
+        if ((q.kind == BC_QUERY_APPROX_T || q.kind == BC_QUERY_HYBRID) && q.T > 0) most += (double)q.T;
+    }
+    const int64_t S = 64 * tile_words_of(g);
+    BCD_TRY(check_graph(g, "bc_batch", ((int64_t)std::min(most, (double)g->n) + S - 1) / S));
     const int64_t launches0 = g->launches;
     bc_batch_info bi;
     memset(&bi, 0, sizeof(bi));
@@ -1748,7 +1762,7 @@ bc_status bc_spd_probe(bc_graph *g, const int32_t *sources, int32_t nsrc, const 
     if (!g || (nsrc > 0 && !sources) || (nt > 0 && !targets))
         return set_error(BC_E_INVALID_ARG, "bc_spd_probe: NULL argument");
     if (nt < 0 || nt > 64) return set_error(BC_E_INVALID_ARG, "bc_spd_probe: 0..64 targets");
-    BCD_TRY(check_graph(g, "bc_spd_probe"));
+    BCD_TRY(check_graph(g, "bc_spd_probe", 1));
     bcd_workspace &ws = g->ws;
     cudaStream_t s = g->stream;
     const int W = tile_words_of(g);  // one tile of the graph's kernel; slots past nsrc stay empty

@@ -345,7 +345,7 @@ extern "C" {
 
 bc_status bc_server_create(bc_graph *g, const bc_server_config *cfg, bc_server **out) {
     if (!g || !out) return set_error(BC_E_INVALID_ARG, "bc_server_create: NULL argument");
-    BCD_TRY(check_graph(g, "bc_server_create"));
+    BCD_TRY(check_graph(g, "bc_server_create", cfg && cfg->tiles_per_slice > 0 ? cfg->tiles_per_slice : 16));
     BCD_TRY(prepare_ordering(g));
     bc_server *s = new bc_server();
     s->g = g;

@@ -1,0 +1,64 @@
+"""What a handle allocates with its calls (unweighted graphs): the state of one
+tile for a call of one tile, of as many tiles as run at once for a later call
+of many. Per vertex and tile in flight the masks, history, chunk lists, levels
+and counts take about 32 S / 4 + 1,000 bytes (S sources a tile), everything
+that is there once less than a tenth of that, and 16 tiles run at once at this
+size: the one-tile call takes less than a quarter of the later one's memory.
+Scores within 1e-9 of the oracle in either order."""
+import pytest
+
+import graphgen as gg
+import oracle as O
+from helpers import close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("acc", [4, 1])
+def test_one_tile_then_many(acc):
+    torch = pytest.importorskip("torch")
+    import paper_1708_08739_gb300 as bcd
+    g = gg.rmat(16, 8, seed=5)
+    og = O.Graph.from_csr(g)
+    r, r2 = (int(x) for x in gg.top_inout_vertices(g, 2))
+    warm = bcd.bc_graph_create(g.n, g.offsets, g.cols)  # modules and the context's own memory
+    bcd.bc_set_config(warm, accumulation=acc)
+    bcd.bc_approx_T(warm, r, 50, 7)
+    bcd.bc_approx_T(warm, r, 8000, 7)
+    warm.close()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    dg = bcd.bc_graph_create(g.n, g.offsets, g.cols)
+    bcd.bc_set_config(dg, accumulation=acc)
+    at = free()
+    used = []
+    for T in (50, 700, 8000, 50):
+        out, info = bcd.bc_batch(dg, [{"r": r, "kind": bcd.BC_QUERY_APPROX_T, "T": T, "seed": 7},
+                                      {"r": r2, "kind": bcd.BC_QUERY_APPROX_T, "T": T, "seed": 7}][: 1 if T == 50 else 2])
+        for q, o in zip((r, r2), out):
+            assert o["status"] == 0 and close(o["bc"], O.bc_approx(og, q, T, 7, 0)[0]), (T, q, o)
+        used.append(at - free())
+    assert info["tiles"] == 1 and used[0] * 4 < used[2] and used[3] == used[2], used
+    dg.close()
+
+
+def test_reach_set_then_probe_then_many():
+    import paper_1708_08739_gb300 as bcd
+    g = gg.rmat(12, 8, seed=12)
+    og = O.Graph.from_csr(g)
+    r = int(gg.top_inout_vertices(g, 1)[0])
+    dg = bcd.bc_graph_create(g.n, g.offsets, g.cols)
+    assert bcd.bc_rv_compute(dg, r).shape[0] == O.rv(og, r).shape[0]
+    bcd.bc_spd_probe(dg, [r], [r])
+    assert close(bcd.bc_exact(dg, r)[0], O.bc_exact(og, r, 0)[0])
+    srv = bcd.Server(dg, tiles_per_slice=1)
+    t = srv.submit({"r": r, "kind": bcd.BC_QUERY_EXACT})
+    x = None
+    while x is None:
+        x = srv.poll(t, timeout_us=100000)
+    srv.close()
+    assert close(x[0]["bc"], O.bc_exact(og, r, 0)[0])
+    dg.close()
