@@ -146,6 +146,7 @@ struct TravParams {
     int64_t pull_arcs_min;
     // tiles
     const int32_t *srcs;  // [ntiles * S], -1 pads the last tile
+    int64_t nsrc;            // occupied slots among the tiles (0: not counted)
     int64_t ntiles;
     // queries (SPD mode); a group holds at most 64 queries (one mask word)
     const uint64_t *qmask;   // [n] bit q set at vertex r_q

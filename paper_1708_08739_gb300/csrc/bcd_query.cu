@@ -1081,6 +1081,7 @@ static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res,
             p.col = g->d_col;
             p.srcs = ws.dlist + (t_lo + first) * S;
             p.ntiles = count;
+            p.nsrc = std::min(nd - (t_lo + first) * S, count * S);
             p.qmask = ws.qmask;
             p.need = ws.need;
             p.exact_q = exact_q;
@@ -1359,6 +1360,7 @@ bc_status run_slice(bc_graph *g, const std::vector<int32_t> &srcs, const std::ve
         p.col = g->d_col;
         p.srcs = ws.dlist + first * S;
         p.ntiles = count;
+        p.nsrc = std::count_if(srcs.begin() + first * S, srcs.begin() + (first + count) * S, [](int32_t v) { return v >= 0; });
         p.qmask = ws.qmask;
         p.need = ws.need;
         p.exact_q = exact_q;

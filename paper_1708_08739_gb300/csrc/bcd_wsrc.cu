@@ -1137,13 +1137,19 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     bcd_workspace &ws = g->ws;
     BCD_TRY(ensure_weighted_state(g));  // ring size, tag array
     BCD_TRY(src_order(g));
-    // blocks by the size of the graph (state is held for that many); a launch
-    // with fewer sources than that takes wider ones
-    const int base_threads = src_threads(g->n);
-    int threads = base_threads;
-    while (threads < kSrcThreads && (int64_t)g->num_sms * (kSrcThreads / (2 * threads)) >= p.ntiles * 64 * W) threads *= 2;
     const int S = 64 * W;
     const int64_t nsrc = p.ntiles * S;
+    // blocks by the size of the graph (state is held for that many); a launch of
+    // fewer sources than that takes wider ones, on small graphs, whose levels
+    // seldom fill more, of 512 threads at most. Empty slots of the last tile do not
+    // count: 64 sources and weights 1..255, 512 / 1024 threads: a 150 x 150 lattice
+    // 41.0 / 44.3 ms, R-MAT graphs of 20,000 vertices 2.06 / 2.04, 65,536 3.51 /
+    // 3.04, 131,072 5.61 / 4.39
+    const int64_t real = p.nsrc > 0 ? p.nsrc : nsrc;
+    const int widest = g->n <= 32 * 1024 ? 512 : kSrcThreads;
+    const int base_threads = src_threads(g->n);
+    int threads = base_threads;
+    while (threads < widest && (int64_t)g->num_sms * (kSrcThreads / (2 * threads)) >= real) threads *= 2;
     const int R = ws.ring;
     // the settled bits join the staging and counters in shared memory while they fit
     const size_t ring = sizeof(WarpArcs) * (size_t)(threads / 32) + sizeof(uint32_t) * 2 * (size_t)R;

@@ -52,3 +52,25 @@ def test_row_lengths(row):
             got, _ = bcd.bc_exact(dg, r)
             assert close(got, O.bc_exact(og, r, 0)[0]), (acc, r)
     dg.close()
+
+
+@pytest.mark.parametrize("n,T,per_sm", [(5000, 64, 2), (32768, 64, 2), (32769, 64, 1), (100_000, 150, 1), (100_000, 400, 2),
+                                        (400_000, 300, 1)])
+def test_few_sources_on_wide_blocks(n, T, per_sm):
+    """A launch of fewer sources than blocks takes wider blocks, fewer per SM;
+    the empty slots of its last tile (up to 255) do not count as sources."""
+    torch = pytest.importorskip("torch")
+    import paper_1708_08739_gb300 as bcd
+    g = gg.erdos_renyi(n, 3 * n, 11)
+    g = g.with_weights(gg.uniform_weights(g.m, 1, 7, 12))
+    og = O.Graph.from_csr(g)
+    dg = bcd.bc_graph_create(g.n, g.offsets, g.cols, g.weights)
+    r = int(gg.top_inout_vertices(g, 1)[0])
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    want = O.bc_approx(og, r, T, 7)[0]
+    for acc in (2, 1):
+        bcd.bc_set_config(dg, accumulation=acc)
+        out, info = bcd.bc_batch(dg, [{"r": r, "kind": bcd.BC_QUERY_APPROX_T, "T": T, "seed": 7}])
+        assert out[0]["status"] == 0 and close(out[0]["bc"], want), (acc, out)
+        assert info["grid_blocks"] == per_sm * sms, (info["grid_blocks"], sms)
+    dg.close()
