@@ -409,7 +409,8 @@ __device__ __forceinline__ void src_finalize(const TravParams &p, const int32_t 
     }
 }
 
-template <class PairT, bool kBits>
+// kFew: every source has a block of its own (see step 1 of a level).
+template <class PairT, bool kBits, bool kFew>
 __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcParams q) {
     extern __shared__ __align__(16) unsigned char s_src[];  // WarpArcs per warp, ring counters, settled bits
     __shared__ int32_t s_ql[64];          // level at which query vertex q settled for this source
@@ -531,17 +532,28 @@ __global__ void __launch_bounds__(kSrcThreads, 1) wsrc_kernel(TravParams p, SrcP
             }
             int *nchp = &s_nch[seg & 1];
             // step 1: the slot's vertices, in groups that the warps draw; their
-            // rows finish here unless they are long
+            // rows finish here unless they are long. In launches of few sources,
+            // whose time is one block's chain of levels, each warp's first group
+            // is fixed, so that on a thin level none draws: all warps on one
+            // counter, most of them to find nothing left, took 3-6 % (64 sources,
+            // 150 x 150 lattice 41.2 -> 39.2 ms, R-MAT 20,000 vertices 2.14 -> 2.06).
+            // Elsewhere the registers that this takes cost more (R-MAT 16 hybrid
+            // batch 58.6 -> 60.0 ms)
             {
                 // one group per warp on a thin level, about two on others
                 const unsigned warps = (unsigned)nwarps;
                 const unsigned share = cnt <= 16 * warps ? (cnt + warps - 1) / warps : (cnt + 2 * warps - 1) / (2 * warps);
                 const int gsize = (int)min(32u, share);
                 const uint32_t *bks = bk + (size_t)slot * (size_t)bcap;
-                for (;;) {
-                    int g0 = 0;
-                    if (lane == 0) g0 = atomicAdd(&s_group, gsize);
-                    g0 = __shfl_sync(kFull, g0, 0);
+                auto draw = [&]() {
+                    int k = 0;
+                    if (lane == 0) k = atomicAdd(&s_group, gsize);
+                    return __shfl_sync(kFull, k, 0);
+                };
+                const int fixed = (int)warps * gsize;  // vertices in the fixed groups
+                auto after = [&]() { return (uint32_t)fixed >= cnt ? (int)cnt : fixed + draw(); };
+                for (int g0 = kFew ? warp * gsize : 0;; g0 = kFew ? after() : 0) {
+                    if (!kFew) g0 = draw();
                     if ((uint32_t)g0 >= cnt) break;
                     // all that a queued vertex needs, in one round of loads
                     int x = 0, seen = 0;
@@ -1143,8 +1155,8 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     // fewer sources than that takes wider ones, on small graphs, whose levels
     // seldom fill more, of 512 threads at most. Empty slots of the last tile do not
     // count: 64 sources and weights 1..255, 512 / 1024 threads: a 150 x 150 lattice
-    // 41.0 / 44.3 ms, R-MAT graphs of 20,000 vertices 2.06 / 2.04, 65,536 3.51 /
-    // 3.04, 131,072 5.61 / 4.39
+    // 39.2 / 41.6 ms, R-MAT graphs of 20,000 vertices 2.06 / 2.04, 65,536 3.47 /
+    // 2.94, 131,072 5.58 / 4.29
     const int64_t real = p.nsrc > 0 ? p.nsrc : nsrc;
     const int widest = g->n <= 32 * 1024 ? 512 : kSrcThreads;
     const int base_threads = src_threads(g->n);
@@ -1156,8 +1168,13 @@ bc_status run_src_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, 
     const size_t done = sizeof(uint32_t) * (((size_t)ws.sheads + 31) / 32);
     const bool bits = ring + done <= kSrcDynSmem;
     const size_t smem = ring + (bits ? done : 0);
-    const void *wide = bits ? (const void *)wsrc_kernel<WidePairs, true> : (const void *)wsrc_kernel<WidePairs, false>;
-    const void *narrow = bits ? (const void *)wsrc_kernel<NarrowPairs, true> : (const void *)wsrc_kernel<NarrowPairs, false>;
+    const bool few = real <= (int64_t)g->num_sms * (kSrcThreads / threads);
+    auto kernel = [&](auto pairs) {
+        using P = decltype(pairs);
+        if (few) return bits ? (const void *)wsrc_kernel<P, true, true> : (const void *)wsrc_kernel<P, false, true>;
+        return bits ? (const void *)wsrc_kernel<P, true, false> : (const void *)wsrc_kernel<P, false, false>;
+    };
+    const void *wide = kernel(WidePairs{}), *narrow = kernel(NarrowPairs{});
     int per_sm = 0, per_sm_n = 0;
     BCD_CUDA(cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     BCD_CUDA(cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

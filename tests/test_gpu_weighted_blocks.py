@@ -74,3 +74,23 @@ def test_few_sources_on_wide_blocks(n, T, per_sm):
         assert out[0]["status"] == 0 and close(out[0]["bc"], want), (acc, out)
         assert info["grid_blocks"] == per_sm * sms, (info["grid_blocks"], sms)
     dg.close()
+
+
+@pytest.mark.parametrize("k", [1, 31, 33, 127, 129, 511, 512, 513, 1023, 1025, 4097])
+def test_level_widths(k):
+    """k vertices that settle at one distance, around the widths at which a
+    block's warps draw further groups: three sources (wide blocks) and the k
+    vertices themselves as sources."""
+    import paper_1708_08739_gb300 as bcd
+    arcs = [(0, 1), (1, 2), (2, 3)] + [(3, 5 + i) for i in range(k)] + [(5 + i, 4) for i in range(k)]
+    arcs += [(4, 5 + k), (5 + k, 6 + k)]
+    g = csr(7 + k, arcs)
+    g = g.with_weights(np.full(g.m, 2, dtype=np.uint32))
+    og = O.Graph.from_csr(g)
+    dg = bcd.bc_graph_create(g.n, g.offsets, g.cols, g.weights)
+    for acc in (1, 2):
+        bcd.bc_set_config(dg, accumulation=acc)
+        for r in (3, 4, 5 + k):
+            got, _ = bcd.bc_exact(dg, r)
+            assert close(got, O.bc_exact(og, r, 0)[0]), (acc, r)
+    dg.close()
