@@ -29,9 +29,8 @@ enum DevErr : int32_t {
 // Per-launch control block of the persistent traversal kernel.
 struct Counters {
     int32_t err;
-    uint32_t bar_count;
-    uint32_t bar_gen;
-    uint32_t pad0;
+    uint32_t bar_count;            // arrivals at the grid's barriers
+    uint32_t pad0[2];
     unsigned long long edges;      // sum over reached (v, s) of out-degree(v)
     unsigned long long levels_max; // deepest level met over all tiles
     unsigned long long ns_fwd;     // block 0's wall time in forward passes
@@ -49,14 +48,14 @@ struct Counters {
     unsigned long long scan_skipped; // ... it was not made, the tile has no result
 };
 
-// Bytes from the counters to the teams' barrier words that follow them.
+// Bytes from the counters to the teams' barrier lines that follow them.
 constexpr size_t kCounterBytes = (sizeof(Counters) + 127) / 128 * 128;
 
-// Barrier words of one team of blocks (unweighted traversal), and its next
+// Barrier count of one team of blocks (unweighted traversal), and its next
 // tile; a cache line each.
 struct __align__(128) TeamBar {
-    uint32_t count;
-    uint32_t gen;
+    uint32_t count;  // arrivals
+    uint32_t pad;
     unsigned long long next;
 };
 

@@ -27,27 +27,23 @@ __device__ __forceinline__ unsigned long long ld_vol(const unsigned long long *p
 
 __device__ __forceinline__ void set_err(Counters *c, int32_t code) { atomicCAS(&c->err, 0, code); }
 
-// Barrier of nb blocks of a cooperative launch, on the words count and gen.
-// Every wait is bounded by timeout_ns of wall time (and a spin cap); on
-// timeout or when another block has flagged an error, returns false and the
-// caller leaves the kernel.
-__device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_ns, uint32_t *count, uint32_t *gens,
-                                    uint32_t nb) {
+// Barrier of nb blocks of a cooperative launch. `count` (zero at launch) only
+// grows, by one per block and barrier, and every block waits until it has
+// passed `target`, this barrier's share, so that the last block to arrive has no
+// words to reset and to release one after the other: those two round trips to L2
+// were a sixth of a thin level (compared modulo 2^32). Every wait is bounded by
+// timeout_ns of wall time (and a spin cap); on timeout or when another block has
+// flagged an error, returns false and the caller leaves the kernel.
+__device__ inline bool grid_barrier(Counters *c, uint32_t &target, double timeout_ns, uint32_t *count, uint32_t nb) {
     __shared__ int s_err;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const uint32_t arrived = nb > 1 ? atomicAdd(count, 1u) : 0u;
-        if (arrived == nb - 1) {
-            if (nb > 1) {
-                atomicExch(count, 0u);
-                __threadfence();
-                atomicExch(gens, gen + 1);
-            }
-        } else {
+        target += nb;
+        if (nb > 1 && atomicAdd(count, 1u) + 1u != target) {
             const unsigned long long t0 = global_ns();
             unsigned long long spins = 0;
-            while (ld_acquire(gens) == gen) {
+            while ((int32_t)(ld_acquire(count) - target) < 0) {
                 if (ld_vol(&c->err) != 0) break;
                 ++spins;
                 if ((double)(global_ns() - t0) > timeout_ns) {
@@ -62,16 +58,15 @@ __device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_n
             }
         }
         __threadfence();
-        gen += 1;
         s_err = ld_vol(&c->err);
     }
     __syncthreads();
     return s_err == 0;
 }
 
-// The same over the whole grid, on the launch's own words.
-__device__ inline bool grid_barrier(Counters *c, uint32_t &gen, double timeout_ns) {
-    return grid_barrier(c, gen, timeout_ns, &c->bar_count, &c->bar_gen, gridDim.x);
+// The same over the whole grid, on the launch's own word.
+__device__ inline bool grid_barrier(Counters *c, uint32_t &target, double timeout_ns) {
+    return grid_barrier(c, target, timeout_ns, &c->bar_count, gridDim.x);
 }
 
 // Start of a tile: thread 0 of each block reads the host's cancel request

@@ -1358,8 +1358,8 @@ __device__ __forceinline__ void load_params(const TravParams &launch, int team) 
 
 // Barrier of the blocks of a team (a lone block needs no wait on others; it
 // still leaves when another team has flagged an error).
-__device__ __forceinline__ bool team_barrier(const TravParams &p, uint32_t &gen) {
-    return grid_barrier(p.ctr, gen, p.timeout_ns, &p.bar->count, &p.bar->gen, (uint32_t)p.team_blocks);
+__device__ __forceinline__ bool team_barrier(const TravParams &p, uint32_t &target) {
+    return grid_barrier(p.ctr, target, p.timeout_ns, &p.bar->count, (uint32_t)p.team_blocks);
 }
 
 template <int W, int MODE, int MINB, typename T>
@@ -1379,7 +1379,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
     const long long nwarps = (long long)p.team_blocks * wpb;
     const long long gthr = (long long)block * blockDim.x + threadIdx.x;
     const long long nthr = (long long)p.team_blocks * blockDim.x;
-    uint32_t gen = 0;
+    uint32_t bar = 0;  // arrivals that the last barrier waited for
     uint64_t *const s_need = tile_need();
     __shared__ int32_t s_minql[S];
     __shared__ uint64_t s_active[W];
@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             s_valid[threadIdx.x] = m;
         }
         warp_buf<W>().st[lane] = Stats();
-        if (!team_barrier(p, gen)) return;
+        if (!team_barrier(p, bar)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
@@ -1462,7 +1462,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             } else {
                 push_masks<W, MODE, kPushU>(L, ccnt, gwarp, nwarps);
             }
-            if (!team_barrier(p, gen)) return;
+            if (!team_barrier(p, bar)) return;
             total = es1;
             const long long enext =
                 (long long)(ld_vol(&p.lev_grab[4 * ((long long)p.maxlev + 2) + L + 1]) & 0xffffffffull);
@@ -1478,7 +1478,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                     gather_level<W, T, kGatherU>(
                         L + 1, ics1, (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + L + 1]), gwarp,
                         nwarps);
-                if (!team_barrier(p, gen)) return;
+                if (!team_barrier(p, bar)) return;
             }
             es_prev = es;
             es = es1;
@@ -1520,13 +1520,13 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                     }
                 }
             }
-            if (!team_barrier(p, gen)) return;
+            if (!team_barrier(p, bar)) return;
         } else if (MODE == kModeScan && !(p.flags & kFlagNoBackward)) {
             if (p.flags & kFlagTrial) {
                 // a lone tile on trial: its terms are counted first, and when they
                 // are too many the tile is left to the Eq. 4 pass
                 scan_count<W>(Lmax, gthr, nthr);
-                if (!team_barrier(p, gen)) return;
+                if (!team_barrier(p, bar)) return;
                 if (scan_too_long(ld_vol(&p.ctr->trial_pairs), ld_vol(&p.ctr->tight))) {
                     if (leader) p.ctr->scan_skipped = 1ull;
                     skipped = true;
@@ -1538,7 +1538,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                 vertex_scan_multi<W, T>(Lmax, gwarp, nwarps);
             else
                 vertex_scan<W, T>(p, Lmax, s_need, gwarp, nwarps);
-            if (!team_barrier(p, gen)) return;
+            if (!team_barrier(p, bar)) return;
         }
         if (MODE == kModeSpd && !(p.flags & kFlagNoBackward)) {
             if (threadIdx.x == 0) s_lstop = 0x7fffffff;
@@ -1574,7 +1574,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                         for (int w = 0; w < W; ++w)
                             atomicOr((unsigned long long *)&row[slot * W + w], (unsigned long long)p.hm[e * W + w]);
                     }
-                    if (!team_barrier(p, gen)) return;
+                    if (!team_barrier(p, bar)) return;
                 }
                 for (int Lb = Lmax; Lb >= lstop; --Lb) {
                     if (threadIdx.x < W) {
@@ -1595,7 +1595,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                         const long long ic = (long long)ld_vol(&p.lev_grab[2 * ((long long)p.maxlev + 2) + Lb]);
                         push_level<W, T>(p, Lb, ics, ic, s_active_next, s_inv, nwarps);
                     }
-                    if (!team_barrier(p, gen)) return;
+                    if (!team_barrier(p, bar)) return;
                 }
             }
         }
@@ -1677,7 +1677,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             }
         }
         if (leader) *(volatile unsigned long long *)&p.bar->next = p.nteams + atomicAdd(&p.ctr->tiles_taken, 1ull);
-        if (!team_barrier(p, gen)) return;
+        if (!team_barrier(p, bar)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
@@ -1851,7 +1851,7 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
             p.npchunks = ws.npchunks;
             p.pull_arcs_min = std::max<int64_t>(1, (int64_t)((double)g->m * g->pull_permille / 1000.0));
         }
-        // the counters and, behind them, the teams' barrier words
+        // the counters and, behind them, the teams' barrier lines
         BCD_CUDA(cudaMemsetAsync(ws.ctr, 0, kCounterBytes + sizeof(TeamBar) * (size_t)ws.teams, g->stream));
         bc_status st = BC_E_INTERNAL;
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;

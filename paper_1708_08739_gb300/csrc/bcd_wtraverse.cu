@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
     const long long LS = (long long)p.maxlev + 2;
     unsigned long long *wl = p.lev_grab;
     unsigned long long *bbase = p.bcount + R;  // consumed entries of each slot
-    uint32_t gen = 0;
+    uint32_t bar = 0;  // arrivals that the last barrier waited for
     WStats st;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
             const int32_t v = tsrc[s];
             s_need[s] = v >= 0 ? p.need[v] : 0ull;
         }
-        if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+        if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                     }
                 }
             }
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
             const long long ecnt = (long long)ld_vol(&p.lev_cnt[seg]);
             const long long ccnt = (long long)ld_vol(&wl[kChunksF * LS + seg]);
             // every block has read the slot's base by now; the new base is
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                     }
                     if (lane < ch.na) st.arcs += (unsigned)((ch.na - lane + 31) / 32);
                 }
-                if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
             }
             es += ecnt;
             ++seg;
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                     p.rsig[v] = p.sigma[iv];
                 }
             }
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
         }
         // ---------------- vertex scan, several query vertices ----------------
         // Column c (query vertex r_c) of a settled pair (t, s) of distance D
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(kFull, pairs, o);
             if (lane == 0 && pairs) atomicAdd(&p.ctr->vpairs, (unsigned long long)pairs);
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
         }
         // ---------------- vertex scan over the settled pairs ----------------
         // A settled pair (t, s) of level sg (distance D) takes the term
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(kFull, pairs, o);
             if (lane == 0 && pairs) atomicAdd(&p.ctr->vpairs, (unsigned long long)pairs);
-            if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+            if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
         }
 
         // ---------------- backward (Eq. 4) over the levels ----------------
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                         }
                     }
                 }
-                if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
                 const long long ccnt = (long long)ld_vol(&wl[kChunksB * LS + sg]);
                 // step 2: chunks of long rows (partial sums indexed by chunk;
                 // an entry's chunks are consecutive); the last chunk of an
@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                             }
                         }
                     }
-                    if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+                    if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
                 }
             }
         }
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
                 for (int i = threadIdx.x; i < 2 * R; i += blockDim.x) p.bcount[i] = 0ull;
             }
         }
-        if (!grid_barrier(p.ctr, gen, p.timeout_ns)) return;
+        if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;
         if (timer) {
             const unsigned long long t = global_ns();
             ns_other += t - t_mark;
