@@ -1438,8 +1438,9 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
                 p.lev_icstart[L + 1] = ics1;
             }
             if (L >= 1) {
+                // the last threads first: on a thin level the first warps push
                 const int nxt = 1 + ((L + 1) & 1);
-                for (long long e = es_prev + gthr; e < es; e += nthr) {
+                for (long long e = es_prev + (nthr - 1 - gthr); e < es; e += nthr) {
                     const int v = p.hv[e];
                     uint64_t *row = p.vs + (size_t)v * p.vs_stride;
 #pragma unroll
