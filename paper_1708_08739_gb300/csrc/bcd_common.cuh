@@ -29,8 +29,8 @@ enum DevErr : int32_t {
 // Per-launch control block of the persistent traversal kernel.
 struct Counters {
     int32_t err;
-    uint32_t bar_count;            // arrivals at the grid's barriers
-    uint32_t pad0[2];
+    uint32_t pad0;
+    unsigned long long bar_count;  // arrivals at the grid's barriers
     unsigned long long edges;      // sum over reached (v, s) of out-degree(v)
     unsigned long long levels_max; // deepest level met over all tiles
     unsigned long long ns_fwd;     // block 0's wall time in forward passes
@@ -54,8 +54,7 @@ constexpr size_t kCounterBytes = (sizeof(Counters) + 127) / 128 * 128;
 // Barrier count of one team of blocks (unweighted traversal), and its next
 // tile; a cache line each.
 struct __align__(128) TeamBar {
-    uint32_t count;  // arrivals
-    uint32_t pad;
+    unsigned long long count;  // arrivals
     unsigned long long next;
 };
 

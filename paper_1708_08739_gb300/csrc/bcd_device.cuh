@@ -13,9 +13,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -29,43 +29,49 @@ __device__ __forceinline__ void set_err(Counters *c, int32_t code) { atomicCAS(&
 
 // Barrier of nb blocks of a cooperative launch. `count` (zero at launch) only
 // grows, by one per block and barrier, and every block waits until it has
-// passed `target`, this barrier's share, so that the last block to arrive has no
-// words to reset and to release one after the other: those two round trips to L2
-// were a sixth of a thin level (compared modulo 2^32). Every wait is bounded by
-// timeout_ns of wall time (and a spin cap); on timeout or when another block has
-// flagged an error, returns false and the caller leaves the kernel.
-__device__ inline bool grid_barrier(Counters *c, uint32_t &target, double timeout_ns, uint32_t *count, uint32_t nb) {
+// reached `target`, so that the last block to arrive has no words to reset and
+// to release one after the other: those two round trips to L2 were a sixth of a
+// thin level. A block that has seen an error (its own, or another's by then)
+// adds kBarError as well, so that all leave at the same barrier without a look
+// at the error word behind it. Every wait is bounded by timeout_ns of wall time
+// (and a spin cap); on timeout or when another block has flagged an error,
+// returns false and the caller leaves the kernel.
+constexpr long long kBarError = 1ll << 48;
+__device__ inline bool grid_barrier(Counters *c, unsigned long long &target, double timeout_ns,
+                                    unsigned long long *count, uint32_t nb) {
     __shared__ int s_err;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        target += nb;
-        if (nb > 1 && atomicAdd(count, 1u) + 1u != target) {
-            const unsigned long long t0 = global_ns();
-            unsigned long long spins = 0;
-            while ((int32_t)(ld_acquire(count) - target) < 0) {
-                if (ld_vol(&c->err) != 0) break;
-                ++spins;
-                if ((double)(global_ns() - t0) > timeout_ns) {
-                    set_err(c, kDevTimeout);
-                    break;
+        bool bad = ld_vol(&c->err) != 0;
+        if (nb > 1) {
+            __threadfence();
+            target += nb;
+            const unsigned long long add = bad ? kBarError + 1 : 1;
+            long long past = (long long)(atomicAdd(count, add) + add - target);  // 0 or more once all have arrived
+            if (past >= 0) {
+                __threadfence();
+            } else {
+                const unsigned long long t0 = global_ns();
+                unsigned long long spins = 0;
+                while ((past = (long long)(ld_acquire(count) - target)) < 0) {
+                    if ((++spins & 3ull) == 0ull && ld_vol(&c->err) != 0) break;
+                    if ((double)(global_ns() - t0) > timeout_ns || spins > (1ull << 31)) {
+                        set_err(c, kDevTimeout);
+                        break;
+                    }
+                    __nanosleep(20);
                 }
-                if (spins > (1ull << 31)) {
-                    set_err(c, kDevTimeout);
-                    break;
-                }
-                __nanosleep(40);
             }
+            bad = past < 0 || past >= kBarError;
         }
-        __threadfence();
-        s_err = ld_vol(&c->err);
+        s_err = bad;
     }
     __syncthreads();
     return s_err == 0;
 }
 
 // The same over the whole grid, on the launch's own word.
-__device__ inline bool grid_barrier(Counters *c, uint32_t &target, double timeout_ns) {
+__device__ inline bool grid_barrier(Counters *c, unsigned long long &target, double timeout_ns) {
     return grid_barrier(c, target, timeout_ns, &c->bar_count, gridDim.x);
 }
 

@@ -1358,7 +1358,7 @@ __device__ __forceinline__ void load_params(const TravParams &launch, int team) 
 
 // Barrier of the blocks of a team (a lone block needs no wait on others; it
 // still leaves when another team has flagged an error).
-__device__ __forceinline__ bool team_barrier(const TravParams &p, uint32_t &target) {
+__device__ __forceinline__ bool team_barrier(const TravParams &p, unsigned long long &target) {
     return grid_barrier(p.ctr, target, p.timeout_ns, &p.bar->count, (uint32_t)p.team_blocks);
 }
 
@@ -1379,7 +1379,7 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
     const long long nwarps = (long long)p.team_blocks * wpb;
     const long long gthr = (long long)block * blockDim.x + threadIdx.x;
     const long long nthr = (long long)p.team_blocks * blockDim.x;
-    uint32_t bar = 0;  // arrivals that the last barrier waited for
+    unsigned long long bar = 0;  // arrivals that the last barrier waited for
     uint64_t *const s_need = tile_need();
     __shared__ int32_t s_minql[S];
     __shared__ uint64_t s_active[W];

@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
     const long long LS = (long long)p.maxlev + 2;
     unsigned long long *wl = p.lev_grab;
     unsigned long long *bbase = p.bcount + R;  // consumed entries of each slot
-    uint32_t bar = 0;  // arrivals that the last barrier waited for
+    unsigned long long bar = 0;  // arrivals that the last barrier waited for
     WStats st;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long t_mark = timer ? global_ns() : 0ull;
