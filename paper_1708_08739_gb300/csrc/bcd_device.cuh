@@ -62,7 +62,8 @@ __device__ inline bool grid_barrier(Counters *c, unsigned long long &target, dou
                     __nanosleep(20);
                 }
             }
-            bad = past < 0 || past >= kBarError;
+            // an error flagged before all have arrived leaves past short of kBarError
+            bad = bad || past < 0 || past >= kBarError / 2;
         }
         s_err = bad;
     }
