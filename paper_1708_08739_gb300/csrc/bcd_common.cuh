@@ -163,7 +163,7 @@ struct TravParams {
     const uint32_t *rwt;     // [m] weights of R(G)'s arcs
     uint64_t *dist;          // [n * S] tentative, then final distances (UINT64_MAX unreached)
     uint32_t *buckets;       // [ring * bcap] queued pairs (vertex << log2 S | source slot), circular per slot
-    unsigned long long *bcount;  // [2 * ring] entries ever queued per slot, then entries consumed per slot
+    unsigned long long *bcount;  // [3 * ring] entries ever queued per slot, entries consumed, distance held plus 1
     int64_t bcap;            // entries per slot (a power of two)
     int32_t ring;            // power of two above the largest weight
     int32_t nw;              // 64-source words of a weighted tile (1, 2, 4, 8 or 16)
@@ -260,7 +260,7 @@ struct bcd_workspace {
     // weighted graphs
     uint64_t *dist = nullptr;     // [n * 64 * W]
     uint32_t *buckets = nullptr;  // [ring * bcap]
-    unsigned long long *bcount = nullptr;  // [2 * ring]
+    unsigned long long *bcount = nullptr;  // [3 * ring]: queued, consumed, distance held plus 1
     int64_t bcap = 0;
     int64_t *lev_dist = nullptr;  // [maxlev + 2]
     int32_t ring = 0;

@@ -267,9 +267,9 @@ static bc_status build_weighted_state(bc_graph *g) {
     ws.bcap = bcap;
     BCD_TRY(dev_alloc(&ws.dist, n * S));
     BCD_TRY(dev_alloc(&ws.buckets, (size_t)R * (size_t)bcap));
-    BCD_TRY(dev_alloc(&ws.bcount, 2 * (size_t)R));
+    BCD_TRY(dev_alloc(&ws.bcount, 3 * (size_t)R));
     BCD_CUDA(cudaMemsetAsync(ws.dist, 0xff, sizeof(uint64_t) * n * S, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 2 * (size_t)R, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 3 * (size_t)R, g->stream));
     const int64_t hneed = std::min<int64_t>((int64_t)(n * S) + 4096, (int64_t)INT32_MAX - 1);
     if (ws.hcap < hneed) BCD_TRY(alloc_history(g, hneed, ws.ccap, ws.pcap, ws.hmcap));
     return BC_OK;
@@ -287,7 +287,7 @@ bc_status grow_buckets(bc_graph *g) {
         free_workspace(g);
         return st;
     }
-    BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 2 * (size_t)ws.ring, g->stream));
+    BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 3 * (size_t)ws.ring, g->stream));
     return BC_OK;
 }
 

@@ -1798,7 +1798,7 @@ bc_status reset_dense_state(bc_graph *g) {
     if (ws.acc) BCD_CUDA(cudaMemsetAsync(ws.acc, 0, sizeof(double) * t * n * 64 * ws.W, g->stream));
     if (ws.dist) {
         BCD_CUDA(cudaMemsetAsync(ws.dist, 0xff, sizeof(uint64_t) * (size_t)ws.n * 64 * ws.W, g->stream));
-        BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 2 * (size_t)ws.ring, g->stream));
+        BCD_CUDA(cudaMemsetAsync(ws.bcount, 0, sizeof(unsigned long long) * 3 * (size_t)ws.ring, g->stream));
     }
     return BC_OK;
 }

@@ -92,12 +92,17 @@ struct Tile {
 };
 
 // Queues the pair (y, s) at tentative distance nd (slot positions wrap
-// around the slot's capacity; overflow is detected when the slot is read).
+// around the slot's capacity; overflow is detected when the slot is read). The
+// slot's tag, nd + 1, tells a block that still looks for the next distance from
+// d which distance the slot holds: blocks ahead of it may be settling d + k by
+// then and queue at d + k + w, which is in the slot of a distance below d + k
+// when k + w reaches R. (A tag not yet written is that of an earlier distance.)
 __device__ __forceinline__ void wenqueue(const TravParams &p, const Tile &t, int y, int s, unsigned long long nd) {
     const int slot = (int)(nd & (unsigned long long)(p.ring - 1));
     const unsigned long long pos = atomicAdd(&p.bcount[slot], 1ull);
     p.buckets[(size_t)slot * p.bcap + (size_t)(pos & (unsigned long long)(p.bcap - 1))] =
         ((uint32_t)y << t.shift) | (uint32_t)s;
+    *(volatile unsigned long long *)(p.bcount + 2 * p.ring + slot) = nd + 1;
 }
 
 // The graph arrays do not change during a launch, so their loads take the
@@ -242,7 +247,8 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
     const int CH = p.chunk_arcs;
     const long long LS = (long long)p.maxlev + 2;
     unsigned long long *wl = p.lev_grab;
-    unsigned long long *bbase = p.bcount + R;  // consumed entries of each slot
+    unsigned long long *bbase = p.bcount + R;      // consumed entries of each slot
+    unsigned long long *btag = p.bcount + 2 * R;   // the distance each slot holds, plus 1 (0: none)
     unsigned long long bar = 0;  // arrivals that the last barrier waited for
     WStats st;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
             __syncthreads();
             for (int k = threadIdx.x + (first ? 0 : 1); k < R; k += blockDim.x) {
                 const int sl = (int)((d + k) & (R - 1));
-                if (ld_vol(&p.bcount[sl]) > ld_vol(&bbase[sl])) {
+                if (ld_vol(&p.bcount[sl]) > ld_vol(&bbase[sl]) && ld_vol(&btag[sl]) == (unsigned long long)(d + k + 1)) {
                     atomicMin(&s_k, k);
                     break;
                 }
@@ -683,7 +689,7 @@ __global__ void __launch_bounds__(512, 2) wtrav_kernel(TravParams p) {
 #pragma unroll
                     for (int k = 0; k < 6; ++k) wl[k * LS + l] = 0ull;
                 }
-                for (int i = threadIdx.x; i < 2 * R; i += blockDim.x) p.bcount[i] = 0ull;
+                for (int i = threadIdx.x; i < 3 * R; i += blockDim.x) p.bcount[i] = 0ull;
             }
         }
         if (!grid_barrier(p.ctr, bar, p.timeout_ns)) return;

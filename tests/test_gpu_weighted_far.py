@@ -44,3 +44,36 @@ def test_long_paths(weight):
     n, dg = path_graph([weight] * 9999)
     check(dg, n, [9000, 5000])
     dg.close()
+
+
+@pytest.mark.parametrize("top", [2, 255, 4095])
+@pytest.mark.parametrize("threads", [128, 512])
+@pytest.mark.parametrize("kernel", [1, 2])
+def test_far_apart_distances(kernel, threads, top):
+    """Few pending vertices with distances up to the largest weight apart, so
+    that a level's offers land in ring slots of smaller distances: every block of
+    the tile kernel (with kernel 2 it runs the query vertices' own traversal) has
+    to find the same next distance, whichever is ahead."""
+    import graphgen as gg
+    import oracle as O
+    import paper_1708_08739_gb300 as bcd
+    rng = np.random.default_rng(top)
+    n, dg = path_graph(rng.integers(max(1, top // 2), top + 1, 250))
+    for acc in (4, 1):
+        bcd.bc_set_config(dg, accumulation=acc, weighted_kernel=kernel, block_threads=threads, weighted_words=1)
+        out, _ = bcd.bc_batch(dg, [{"r": r} for r in (30, 230)])
+        for r, o in zip((30, 230), out):
+            assert o["status"] == 0 and close(o["bc"], r * (n - 1 - r)), (acc, r, o)
+        assert close(bcd.bc_exact(dg, 60)[0], 60 * (n - 61)), acc
+    dg.close()
+    g = gg.erdos_renyi(500, 700, 4)
+    g = g.with_weights(gg.uniform_weights(g.m, max(1, top // 2), top, 3))
+    og = O.Graph.from_csr(g)
+    dg = bcd.bc_graph_create(g.n, g.offsets, g.cols, g.weights)
+    rs = [int(x) for x in gg.top_inout_vertices(g, 2)]
+    for acc in (4, 1):
+        bcd.bc_set_config(dg, accumulation=acc, weighted_kernel=kernel, block_threads=threads)
+        out, _ = bcd.bc_batch(dg, [{"r": r} for r in rs])
+        for r, o in zip(rs, out):
+            assert o["status"] == 0 and close(o["bc"], O.bc_exact(og, r, 0)[0]), (acc, r)
+    dg.close()
