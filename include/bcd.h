@@ -211,8 +211,10 @@ typedef struct {
     int64_t union_arcs;       /* sum over tiles of the out-arcs of those vertices */
     int64_t scan_pairs;       /* accumulation 2: (t, s) pairs with the query vertex on a
                                  shortest s-t path (the terms of the vertex scan) */
-    double ms_root;           /* accumulation 2: CUDA-event time of the traversal from the
-                                 query vertex (inside ms_spd, not in ms_traversal) */
+    double ms_root;           /* vertex scan: CUDA-event time of the traversal from the query
+                                 vertices (inside ms_spd, not in ms_traversal). The handle
+                                 keeps the last one: 0 when the scan before was at the same
+                                 vertices in the same order */
     int64_t pull_levels;      /* forward levels run bottom-up (bc_config.pull_permille) */
     int64_t scan_tiles;       /* tiles whose dependencies came from the vertex scan */
     int64_t eq4_reached_pairs; /* reached_pairs and tight_pairs of the tiles that ran the */
@@ -275,8 +277,9 @@ bc_status bc_spd_probe(bc_graph *g, const int32_t *sources, int32_t nsrc, const 
  * max_device_bytes; otherwise it returns to the head of the queue until
  * running queries free their bytes, and a query whose bytes alone exceed the
  * budget completes with status BC_E_BUSY. The per-(vertex, source) slabs
- * (sigma, accumulators, masks, level history) are allocated once per graph
- * for one tile and shared by all tiles, outside the budget. An admitted
+ * (sigma, accumulators, masks, level history) belong to the graph, for as many
+ * tiles as run at once, and are outside the budget; counts and accumulators
+ * are allocated by the first slice that needs them. An admitted
  * query's sources join the pool of pending sources: a source already pending
  * for another query is run once for both. The worker runs the pool in slices
  * of tiles_per_slice tiles, taking sources round-robin across the active

@@ -129,10 +129,8 @@ struct TravParams {
     int32_t *pdone;     // [pcap]
     int64_t pcap;
     unsigned long long *lev_cnt;   // [maxlev + 2]
-    unsigned long long *lev_ccnt;  // [maxlev + 2]
     unsigned long long *lev_grab;  // [6 * (maxlev + 2)] hand-out counters and counts, see bcd_workspace
     int64_t *lev_start;            // [maxlev + 2]
-    int64_t *lev_cstart;           // [maxlev + 2]
     int64_t *lev_icstart;          // [maxlev + 2] first in-arc chunk of each level
     int32_t maxlev;
     int32_t pad1;
@@ -241,11 +239,9 @@ struct bcd_workspace {
     int32_t *pdone = nullptr;
     int64_t pcap = 0;
     unsigned long long *lev_cnt = nullptr;
-    unsigned long long *lev_ccnt = nullptr;
     unsigned long long *lev_grab = nullptr;  // [6 * (maxlev + 2)]: forward and backward hand-out, in-arc chunk
                                              // counts, frontier out-arc sums, entries | chunks << 32, gather hand-out
     int64_t *lev_start = nullptr;
-    int64_t *lev_cstart = nullptr;
     int64_t *lev_icstart = nullptr;
     int32_t maxlev = 0;
     int2 *pchunks = nullptr;      // in-arc chunks of every vertex (bottom-up levels), unweighted graphs

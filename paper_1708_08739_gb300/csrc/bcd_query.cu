@@ -211,23 +211,18 @@ static bc_status alloc_history(bc_graph *g, int64_t hcap, int64_t ccap, int64_t 
 bc_status alloc_levels(bc_graph *g, int64_t maxlev) {
     bcd_workspace &ws = g->ws;
     dev_free(ws.lev_cnt);
-    dev_free(ws.lev_ccnt);
     dev_free(ws.lev_grab);
     dev_free(ws.lev_start);
-    dev_free(ws.lev_cstart);
     dev_free(ws.lev_icstart);
     dev_free(ws.lev_dist);
     ws.maxlev = (int32_t)maxlev;
     const size_t L = ((size_t)maxlev + 2) * (size_t)ws.teams;
     BCD_TRY(dev_alloc(&ws.lev_cnt, L));
-    BCD_TRY(dev_alloc(&ws.lev_ccnt, L));
     BCD_TRY(dev_alloc(&ws.lev_grab, 6 * L));
     BCD_TRY(dev_alloc(&ws.lev_start, L));
-    BCD_TRY(dev_alloc(&ws.lev_cstart, L));
     BCD_TRY(dev_alloc(&ws.lev_icstart, L));
     if (g->weighted) BCD_TRY(dev_alloc(&ws.lev_dist, L));
     BCD_CUDA(cudaMemsetAsync(ws.lev_cnt, 0, sizeof(unsigned long long) * L, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.lev_ccnt, 0, sizeof(unsigned long long) * L, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.lev_grab, 0, sizeof(unsigned long long) * 6 * L, g->stream));
     return BC_OK;
 }
@@ -347,10 +342,8 @@ void free_workspace(bc_graph *g) {
     dev_free(ws.partial);
     dev_free(ws.pdone);
     dev_free(ws.lev_cnt);
-    dev_free(ws.lev_ccnt);
     dev_free(ws.lev_grab);
     dev_free(ws.lev_start);
-    dev_free(ws.lev_cstart);
     dev_free(ws.lev_icstart);
     dev_free(ws.pchunks);
     dev_free(ws.rvmask);
@@ -878,13 +871,12 @@ static void shard_tiles(int64_t ntiles, int32_t k, int32_t nshards, int64_t *lo,
     *hi = ntiles * (k + 1) / nshards;
 }
 
-// Runs one group of at most 64 queries whose out-degree is positive; with
-// nshards > 1 only the group's tiles of shard k run, and each score is that
-// shard's part of the sum (already scaled by |RV| / T for sampled queries).
 // The traversal from the query vertices that the vertex scan reads: from one
 // vertex (rlev, rsig) or from several columns (rlevq, rsigq, with the column
-// tables qcol / croot staged in the small buffer). Kept across calls while the
-// ordered list of vertices is unchanged (it depends on the graph only).
+// tables qcol / croot staged in the small buffer). It depends on the graph and
+// the ordered list of vertices alone, and the handle keeps the last one: the
+// slices of a served query and repeated questions about the same vertices (other
+// eps, T or seeds) share it. A call at other vertices runs its own.
 static bc_status scan_roots(bc_graph *g, const std::vector<int32_t> &roots, const std::vector<int32_t> &qcol,
                             double *ms_root) {
     bcd_workspace &ws = g->ws;
@@ -911,6 +903,9 @@ static bc_status scan_roots(bc_graph *g, const std::vector<int32_t> &roots, cons
     return BC_OK;
 }
 
+// Runs one group of at most 64 queries whose out-degree is positive; with
+// nshards > 1 only the group's tiles of shard k run, and each score is that
+// shard's part of the sum (already scaled by |RV| / T for sampled queries).
 static bc_status run_group(bc_graph *g, std::vector<GQuery> &qs, bc_result *res, GroupTimes &tm, int32_t shard,
                            int32_t nshards) {
     bcd_workspace &ws = g->ws;

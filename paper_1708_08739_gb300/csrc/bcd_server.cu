@@ -60,8 +60,9 @@ double samples_for(double eps, double delta) { return std::ceil(std::log(2.0 / d
 // (8 bytes) and, for a sampled query, its row of draw counts (64 x 4 bytes);
 // per tile of S sources, the tile's per-query partial sums (64 x 8 bytes).
 // The per-(vertex, source) slabs (sigma, accumulators, masks, level history)
-// are allocated once per graph for one tile and reused by every tile, so they
-// are the server's fixed cost, outside the budget.
+// belong to the graph, for as many tiles as run at once, and are reused by every
+// tile, so they are the server's fixed cost, outside the budget (the counts and
+// accumulators come with the first slice that needs them).
 int64_t bcd_staged_bytes(int64_t sources, bool sampled, int S) {
     const int64_t per = 4 + 8 + (sampled ? 64 * 4 : 0);
     return sources * per + (sources + S - 1) / S * 64 * 8;

@@ -428,7 +428,6 @@ __device__ void init_tile(const TravParams &p, const int32_t *tsrc) {
     __syncthreads();
     if (t == 0) {
         p.lev_cnt[0] = (unsigned long long)s_valid;
-        p.lev_ccnt[0] = (unsigned long long)s_scan[S - 1];
         p.lev_grab[4 * ((long long)p.maxlev + 2)] = (unsigned long long)s_valid | ((unsigned long long)s_scan[S - 1] << 32);
     }
 }
@@ -1342,10 +1341,8 @@ __device__ __forceinline__ void load_params(const TravParams &launch, int team) 
         p.chunks += t * (size_t)p.ccap;
         p.ichunks += t * (size_t)p.ccap;
         p.lev_cnt += t * lev;
-        p.lev_ccnt += t * lev;
         p.lev_grab += t * 6 * lev;
         p.lev_start += t * lev;
-        p.lev_cstart += t * lev;
         p.lev_icstart += t * lev;
         p.qlevel += t * ws * 64;
         p.dep += t * ws * 64;
@@ -1429,11 +1426,8 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             const long long es1 = es + ecnt, cs1 = cs + ccnt, ics1 = ics + iccnt;
             if (leader) {
                 p.lev_cnt[L] = (unsigned long long)ecnt;  // published for the passes after the forward
-                p.lev_ccnt[L] = (unsigned long long)ccnt;
                 p.lev_start[L] = es;
-                p.lev_cstart[L] = cs;
                 p.lev_start[L + 1] = es1;
-                p.lev_cstart[L + 1] = cs1;
                 p.lev_icstart[L] = ics;
                 p.lev_icstart[L + 1] = ics1;
             }
@@ -1667,7 +1661,6 @@ __global__ void __launch_bounds__(512, MINB) trav_kernel(const __grid_constant__
             if (block == 0) {
                 for (int l = threadIdx.x; l <= Lmax + 1; l += blockDim.x) {
                     p.lev_cnt[l] = 0ull;
-                    p.lev_ccnt[l] = 0ull;
                     p.lev_grab[l] = 0ull;
                     p.lev_grab[p.maxlev + 2 + l] = 0ull;
                     p.lev_grab[2 * (p.maxlev + 2) + l] = 0ull;
@@ -1792,7 +1785,6 @@ bc_status reset_dense_state(bc_graph *g) {
         ws.sigma_zero = true;
     }
     BCD_CUDA(cudaMemsetAsync(ws.lev_cnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
-    BCD_CUDA(cudaMemsetAsync(ws.lev_ccnt, 0, sizeof(unsigned long long) * t * lev, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.lev_grab, 0, sizeof(unsigned long long) * t * 6 * lev, g->stream));
     BCD_CUDA(cudaMemsetAsync(ws.pdone, 0, sizeof(int32_t) * (size_t)(g->weighted ? ws.pcap : 1), g->stream));
     if (ws.acc) BCD_CUDA(cudaMemsetAsync(ws.acc, 0, sizeof(double) * t * n * 64 * ws.W, g->stream));
@@ -1834,10 +1826,8 @@ bc_status run_traversal(bc_graph *g, int W, TravParams &p, int *levels_out, unsi
         p.pdone = ws.pdone;
         p.pcap = ws.pcap;
         p.lev_cnt = ws.lev_cnt;
-        p.lev_ccnt = ws.lev_ccnt;
         p.lev_grab = ws.lev_grab;
         p.lev_start = ws.lev_start;
-        p.lev_cstart = ws.lev_cstart;
         p.lev_icstart = ws.lev_icstart;
         p.maxlev = ws.maxlev;
         p.ctr = ws.ctr;

@@ -17,7 +17,7 @@
 // with the start and distance of each distance level; and the bucket ring: R
 // slots (R a power of two above the largest weight) of bcap queued vertices
 // each, with their queued / consumed counters in shared memory. Eq. 4
-// launches also keep one bit per arc (see src_relax).
+// launches also keep one bit per arc (see src_offers).
 //
 // The state is indexed by position, not by vertex: positions sort the vertices
 // by their in-degree's power of two, largest first (src_order). A relaxation
