@@ -44,13 +44,14 @@ WORKLOAD = "rmat22_ef8_recip30_sampled64"
 
 # DRAM bytes per (source, reached arc) of the batched traversal kernel
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch over the edges it
-# traversed), measured with ncu on a small launch of the same kernel (one
-# sampled query, 512 draws, on the R-MAT scale 20 graph: --case profile) and
+# traversed), measured with ncu on a small launch of the same kernel and path
+# (eight query vertices, 510 sources, the scan over several vertices, on the
+# R-MAT scale 20 graph: --case profile --case-queries 8 --accumulation 3) and
 # scaled to the bench's launch by its edge count. The figure belongs to the
 # kernel sources it was taken on: when their hash differs, traffic is null.
 KERNEL_SOURCES = ["bcd_traverse.cu", "bcd_device.cuh", "bcd_common.cuh"]
-TRAFFIC = {"sources_sha256": "6450effc35581c4c301354863a5199a3480ebe128e9b6da6da80517b68ed4363",
-           "bytes_per_reached_arc": 6.266, "tile_words": 4}
+TRAFFIC = {"sources_sha256": "9dd92c67eb7134866b136d810e309559034caffc165d3451ce576f1936e29288",
+           "bytes_per_reached_arc": 1.694, "tile_words": 4}
 
 
 def log(*a):
